@@ -112,6 +112,8 @@ struct LaunchArgs {
 int launch_simt_tri(const LaunchArgs& a, int precision, bool assemble);
 int launch_simt_tet_mass(const LaunchArgs& a, int precision, bool assemble);
 int launch_simt_tet_poisson(const LaunchArgs& a, int precision, bool assemble);
+// FP64 Poisson (every degree, triangles and tetrahedra), contracted in fixed point
+int launch_poisson_fixed(const LaunchArgs& a, bool assemble);
 int launch_simt_vector(const LaunchArgs& a, int precision, bool assemble);
 int launch_simt_source(const LaunchArgs& a, int precision, bool assemble);
 int launch_tc(const LaunchArgs& a, int precision, bool assemble);

@@ -1,0 +1,107 @@
+// FP64 contractions in 64-bit integer arithmetic.
+//
+// GB300 has two FP64 lanes per SM and clock against 64 or more 32-bit integer
+// multiply-add lanes, so a contraction sum_k a_k g_k whose factors are known once per row
+// (a) and once per cell (g) is taken in fixed point: each factor is an integer of B bits
+// times a power of two, the power shared by a row or by a cell, and the products are
+// summed exactly in two 64-bit integers, then rounded once to FP64.
+//
+//   x = f 2^(e - B),  |x| < 2^e,  f = h 2^29 + l,  -2^28 <= l < 2^28,  |h| <= 2^(B - 29)
+//   sum a g = 2^(ea + eg + 58 - 2B) [ sum ah gh + 2^-29 sum (ah gl + al gh) + ... ]
+//
+// (three 32 x 32 -> 64 multiply-adds per term; the dropped al gl terms are below
+// 2^(56 - 2B) of the scales each). Both sums stay within 63 bits for K 4^(B - 29) < 2^63:
+// B = 59 for K <= 7, B = 58 for K <= 31. Rounding the factors and dropping al gl costs at
+// most K 2^-B of 2^(ea + eg) in all; FP64 multiply-adds cost K 2^-53 of the partial sums.
+// The fixed point is thus the more accurate one wherever the partial sums are not more
+// than 2^(B - 53) below the scales, which the callers ensure by a condition on the cell
+// (its geometry factors of comparable size); other cells take the FP64 multiply-adds.
+#pragma once
+
+#include <cuda_runtime.h>
+
+namespace ffc {
+
+// |x| < 2^fix_exponent(x) for finite x; 1025 for infinities and NaN
+__device__ __forceinline__ int fix_exponent(double x) {
+  return int((unsigned(__double2hiint(x)) >> 20) & 0x7ffu) - 1022;
+}
+
+// x 2^(B - e) rounded to the nearest integer (halves away from zero), |x| < 2^e
+template <int B>
+__device__ __forceinline__ long long fix_round(double x, int e) {
+  const unsigned hw = unsigned(__double2hiint(x));
+  const int ex = int((hw >> 20) & 0x7ffu);
+  unsigned long long m = (static_cast<unsigned long long>(hw & 0xfffffu) << 32) | unsigned(__double2loint(x));
+  if (ex) m |= 1ull << 52;
+  const int sh = (ex ? ex : 1) - 1075 + B - e;  // x = +-m 2^(ex - 1075)
+  unsigned long long f;
+  if (sh >= 0) f = m << (sh < 63 ? sh : 63);
+  else f = -sh < 64 ? (m + (1ull << (-sh - 1))) >> -sh : 0ull;
+  return (hw >> 31) ? -static_cast<long long>(f) : static_cast<long long>(f);
+}
+
+// The two parts (h, l) of a fixed-point factor. The empty asm hides that they came from a
+// 64-bit value: otherwise the compiler keeps the sign-extended value across a loop and
+// multiplies 64 x 64 bits (four multiply-adds for one).
+__device__ __forceinline__ int2 fix_split(long long f) {
+  const long long h64 = (f + (1ll << 28)) >> 29;
+  int h = int(h64), l = int(f - (h64 << 29));
+  asm("" : "+r"(h), "+r"(l));
+  return make_int2(h, l);
+}
+template <int B>
+__device__ __forceinline__ int2 fix_parts(double x, int e) {
+  return fix_split(fix_round<B>(x, e));
+}
+
+// The two partial sums of a contraction; `mid` starts at half a unit of the final shift.
+struct FixAcc {
+  long long hi = 0, mid = 1ll << 28;
+  __device__ __forceinline__ void add(int2 a, int2 g) {
+    hi += static_cast<long long>(a.x) * g.x;
+    mid += static_cast<long long>(a.x) * g.y;
+    mid += static_cast<long long>(a.y) * g.x;
+  }
+  __device__ __forceinline__ long long sum() const { return hi + (mid >> 29); }
+};
+
+// v 2^ulog rounded to the nearest double, |v| < 2^63, for results with normal exponents;
+// `e20` is ulog << 20. Two forms, which a kernel can mix so that two pipes share the work.
+//
+// On the integer pipes: the magnitude is normalised to a leading one at bit 63 and cut to
+// 53 bits, and the next bit (halves away from zero) and (exponent - 1) << 52 are added: the
+// leading one completes the exponent field, and so does a carry of the rounding.
+__device__ __forceinline__ double fix_to_double(long long v, int e20) {
+  const long long s = v >> 63;
+  const unsigned long long m = static_cast<unsigned long long>((v ^ s) - s);
+  unsigned mh = unsigned(m >> 32), ml = unsigned(m);
+  int expo = e20 + (1085 << 20);
+  if (mh == 0) {
+    mh = ml;
+    ml = 0;
+    expo -= 32 << 20;
+  }
+  const unsigned sh = unsigned(__clz(int(mh)));  // 32 only for zero
+  const unsigned nh = __funnelshift_l(ml, mh, sh), nl = ml << (sh & 31u);
+  const unsigned up = (nl >> 10) & 1u;
+  const unsigned lo = __funnelshift_r(nl, nh, 11) + up;
+  unsigned hi = (nh >> 11) + (lo < up ? 1u : 0u) + (unsigned(expo) - (sh << 20));
+  if (mh == 0) hi = 0;  // then lo is 0 too
+  return __hiloint2double(int(hi | (unsigned(s >> 32) & 0x80000000u)), int(lo));
+}
+
+// On the FP64 pipe: the top 52 bits and the low 12 are placed in the significands of two
+// doubles of fixed exponent (T = 1.5 2^52 u + top u with u = 2^(ulog + 12), and L = 2^52
+// 2^ulog + low 2^ulog), so T - (1.5 2^52 + 2^40) u = top u - 2^52 2^ulog is exact and
+// adding L rounds once: two FP64 additions and no normalisation.
+__device__ __forceinline__ double fix_to_double_fp64(long long v, int e20) {
+  const long long top = v >> 12;
+  const int base = e20 + (1087 << 20);
+  const double T = __hiloint2double(int(top >> 32) + base + 0x80000, int(top));
+  const double c = __hiloint2double(base + 0x80100, 0);
+  const double L = __hiloint2double(e20 + (1075 << 20), int(v) & 0xfff);
+  return (T - c) + L;
+}
+
+}  // namespace ffc

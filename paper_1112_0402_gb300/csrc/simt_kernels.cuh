@@ -34,11 +34,12 @@ struct SimtCfg {
   static constexpr int VEC = 16 / int(sizeof(T));
   static constexpr int NAP = (NA + VEC - 1) / VEC * VEC;
   static constexpr int RMAX_THREADS = BLOCK > 0 ? BLOCK : 512;
-  // symmetric forms on the FP64 pipe contract only the entries i1 <= i2 (Section 3.5:
-  // a symmetric form needs fewer operations) and store each result at (i1, i2) and
+  // dense elasticity on the FP64 pipe contracts only the entries i1 <= i2 (Section 3.5:
+  // a symmetric form needs fewer operations) and stores each result at (i1, i2) and
   // (i2, i1); the FP32 paths stay HBM-bound on stores and keep the full, coalesced layout
+  // (the FP64 Poisson form has its own kernel, poisson_fixed.cu)
   static constexpr bool SYMM =
-      BLOCK == 0 && sizeof(T) == 8 && (FORM == FFC_POISSON || FORM == FFC_ELASTICITY);
+      BLOCK == 0 && sizeof(T) == 8 && FORM == FFC_ELASTICITY;
   static constexpr int NE = SYMM ? N * (N + 1) / 2 : NN;  // entries contracted per cell
   // FP32 tabulate of the Poisson form with element tensors of 256 entries or more made of
   // whole 16-byte groups (P3 on tetrahedra): a thread owns four consecutive entries of each

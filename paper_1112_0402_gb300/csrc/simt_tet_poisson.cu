@@ -1,4 +1,4 @@
-// CUDA-core kernels: Poisson on tetrahedra, P1..P4.
+// CUDA-core kernels: Poisson on tetrahedra, P1..P4 (FP64: poisson_fixed.cu).
 #include <type_traits>
 
 #include "simt_dispatch.cuh"
@@ -6,6 +6,7 @@
 namespace ffc {
 int launch_simt_tet_poisson(const LaunchArgs& a, int precision, bool assemble) {
   if (a.f->d != 3 || a.f->kind != FFC_POISSON) return FFC_EUNSUPPORTED;
-  return simt_by_precision<3, FFC_POISSON, 4>(a, precision, assemble);
+  if (precision == FFC_FP64) return launch_poisson_fixed(a, assemble);
+  return precision == FFC_FP32 ? simt_by_degree<3, FFC_POISSON, 4, float>(a, assemble) : FFC_EUNSUPPORTED;
 }
 }  // namespace ffc
