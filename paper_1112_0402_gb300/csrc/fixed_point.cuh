@@ -55,15 +55,17 @@ __device__ __forceinline__ int2 fix_parts(double x, int e) {
   return fix_split(fix_round<B>(x, e));
 }
 
-// The two partial sums of a contraction; `mid` starts at half a unit of the final shift.
+// The partial sums of a contraction, the middle one in two chains (a chain's latency, not
+// the multipliers, would bound a thread otherwise); `mid` starts at half a unit of the
+// final shift.
 struct FixAcc {
-  long long hi = 0, mid = 1ll << 28;
+  long long hi = 0, mid = 1ll << 28, mid2 = 0;
   __device__ __forceinline__ void add(int2 a, int2 g) {
     hi += static_cast<long long>(a.x) * g.x;
     mid += static_cast<long long>(a.x) * g.y;
-    mid += static_cast<long long>(a.y) * g.x;
+    mid2 += static_cast<long long>(a.y) * g.x;
   }
-  __device__ __forceinline__ long long sum() const { return hi + (mid >> 29); }
+  __device__ __forceinline__ long long sum() const { return hi + ((mid + mid2) >> 29); }
 };
 
 // v 2^ulog rounded to the nearest double, |v| < 2^63, for results with normal exponents;

@@ -18,6 +18,15 @@
 // 27x (convection) and 9x (elasticity) fewer multiply-adds and a reference tensor small
 // enough for registers.
 //
+// The FP64 contraction runs in fixed point (fixed_point.cuh): with FP64 multiply-adds it
+// held the FP64 pipe at 94% with the issue slots at 9%. Now the wide integer multiply-adds
+// (convection P2: 90 per value, 360 SM clocks a cell against 306 for its A_K at the HBM
+// rate), their latency at two resident CTAs and the geometry phase bound it. FP64
+// multiply-adds -> fixed point: tabulate convection P2 on 384,000 tets 2309 -> 816 us, P1
+// 240 -> 175; elasticity P3 on 48,000 tets 3180 -> 900, P2 on 162,000 2605 -> 794, P1 on
+// 384,000 1183 -> 499; assembly of 82,944 tets, convection P2 570 -> 267, elasticity P2
+// 1508 -> 477 us.
+//
 // Thread layouts. Elasticity, "row slots": a slot is (s1, c2, s2), numbered with s2
 // fastest, then c2, then s1, so consecutive slots are consecutive entries of element
 // tensor row (c1, s1) for every c1; the slot keeps R[(s1,s2)] in registers and per cell
@@ -36,6 +45,7 @@
 #include <type_traits>
 
 #include "ffc_internal.h"
+#include "fixed_point.cuh"
 #include "geometry.cuh"
 #include "simt_kernels.cuh"
 
@@ -64,25 +74,39 @@ struct BlockCfg {
   static constexpr int GRP = NT >= NSL ? NT / NSL : 1;  // thread groups; a tile's cells are dealt to them
   static constexpr int PPT = (NSL + NT - 1) / NT;       // slots per thread
   static constexpr bool REG_R = PPT * KR * int(sizeof(T)) / 4 <= 64;
-  static constexpr int E_DEF = (FORM == FFC_NS_CONVECTION && sizeof(T) == 8) ? 64 : 128;
+  static constexpr int E_DEF = sizeof(T) == 8 ? 64 : 128;
   static constexpr int E = KE_T > 0 ? (KE_T * GRP < 128 ? KE_T * GRP : 128) : E_DEF;  // cells per tile
   static constexpr int NCOEF = FORM == FFC_NS_CONVECTION ? N : 0;
   static constexpr size_t G_BYTES = size_t(E) * NB * KRP * sizeof(T);
   static constexpr size_t R_BYTES = REG_R ? 0 : size_t(NP2) * KRP * sizeof(T);
   static constexpr size_t W_BYTES = size_t(E) * NCOEF * sizeof(double);
-  static constexpr size_t SMEM = G_BYTES + R_BYTES + W_BYTES;
+  // FP64 contracts in fixed point (fixed_point.cuh): the geometry blocks and the reduced
+  // rows are kept as fixed-point parts, with an exponent per cell and per slot
+  static constexpr bool FIX = sizeof(T) == 8;
+  static constexpr int BITS = 58;       // KR <= 31 terms
+  // FP64 scratch per cell: J^-1, |det J| and, for elasticity, |det J| mu K K^T (symmetric)
+  static constexpr int XD = D * D + 1 + (DIAG ? 0 : D * (D + 1) / 2);
+  static constexpr size_t X_BYTES = FIX ? size_t(E) * (XD * sizeof(double) + 4 * sizeof(int)) : 0;
+  static constexpr size_t SMEM = G_BYTES + R_BYTES + W_BYTES + X_BYTES;
   // register budget of the single-form FP32 kernel: two resident CTAs of 257..511 threads
-  // (up to 78 registers), three of up to 256; FP64 (bound by the FP64 pipe) keeps its
-  // reduced rows in registers without spills
+  // (up to 78 registers), three of up to 256; FP64 keeps its reduced rows in registers
+  // without spills (a bound for two CTAs: elasticity P3 1262 against 945 us; for three:
+  // convection P2 986 against 816 us)
   static constexpr int MIN_BLOCKS = sizeof(T) == 8 ? 1 : (NT >= 512 ? 1 : (NT > 256 ? 2 : 3));
 };
 
 template <class C, typename T>
 struct BlockRows {
-  T rr[C::REG_R ? C::PPT : 1][C::REG_R ? C::KR : 1];  // reduced rows of the thread's slots
+  using V = typename std::conditional<C::FIX, int2, T>::type;
+  V rr[C::REG_R ? C::PPT : 1][C::REG_R ? C::KR : 1];  // reduced rows of the thread's slots
+  int expo[C::FIX ? C::PPT : 1];                      // FP64: exponents of the results (<< 20)
 };
 
-// Tabulate of the single-form FP32 convection kernel: the element tensors of CELLS cells
+// Sentinel exponent of a cell whose geometry blocks stay doubles (exponents are stored
+// shifted into a double's exponent field, multiples of 2^20).
+constexpr int BLOCK_FIX_NONE = 1;
+
+// Tabulate of the single-form convection kernels: the element tensors of CELLS cells
 // at a time are put together in shared memory (the off-diagonal blocks, always zero, are
 // written there once), then one thread writes them to A_K with a TMA bulk copy, two
 // buffers deep, so A_K leaves the SM as whole contiguous lines instead of runs of n_s
@@ -92,7 +116,7 @@ struct BlockRows {
 // row, writes directly (staged in 2-cell chunks its P3 tabulate went 0.513 -> 0.608 ms).
 template <class C, typename T, bool ASSEMBLE>
 struct BlockStaging {
-  static constexpr bool ON = !ASSEMBLE && C::DIAG && sizeof(T) == 4;
+  static constexpr bool ON = !ASSEMBLE && C::DIAG;
   static constexpr int CELLS = C::GRP > 4 ? C::GRP : 4;  // at least one cell per thread group
   static constexpr size_t BUF = size_t(CELLS) * C::NN * sizeof(T);  // a multiple of 16 bytes
   static constexpr size_t BYTES = ON ? 2 * BUF : 0;
@@ -140,8 +164,16 @@ __device__ __forceinline__ void block_rows_init(const void* r, BlockRows<C, T>& 
     for (int j = 0; j < C::PPT; ++j) {
       const int q = slot_of<C>(t, j);
       const int pp = q >= 0 ? pair_of_slot<C>(q) : 0;
+      if constexpr (C::FIX) {
+        int e = -1022;
+        for (int k = 0; k < C::KR; ++k) e = max(e, fix_exponent(Rg[size_t(pp) * C::KR + k]));
 #pragma unroll
-      for (int k = 0; k < C::KR; ++k) b.rr[j][k] = q >= 0 ? Rg[size_t(pp) * C::KR + k] : T(0);
+        for (int k = 0; k < C::KR; ++k) b.rr[j][k] = fix_parts<C::BITS>(Rg[size_t(pp) * C::KR + k], e);
+        b.expo[j] = (e + 58 - 2 * C::BITS) * (1 << 20);
+      } else {
+#pragma unroll
+        for (int k = 0; k < C::KR; ++k) b.rr[j][k] = q >= 0 ? Rg[size_t(pp) * C::KR + k] : T(0);
+      }
     }
   } else {
     T* Rs = reinterpret_cast<T*>(smem + C::G_BYTES);
@@ -149,6 +181,112 @@ __device__ __forceinline__ void block_rows_init(const void* r, BlockRows<C, T>& 
       const int rw = k / C::KRP, kk = k % C::KRP;
       Rs[k] = kk < C::KR ? Rg[size_t(rw) * C::KR + kk] : T(0);
     }
+  }
+}
+
+// FP64: the geometry blocks of a tile's cells in fixed point. One thread per cell forms
+// J^-1 and |det J|; then the whole CTA forms the blocks, one (cell, node) or (cell, c1, c2)
+// part at a time, with the cell's largest exponent in shared memory, and rewrites them in
+// place as fixed-point parts. (One thread per cell for all of it left five of seven warps
+// waiting: convection P2 881 against 816 us.)
+//
+// Fixed point where every row's scale is within 2^3 (convection: the rows K_a; an entry
+// errs by below 2^-53 of the smallest row's largest terms) or 2^6 (elasticity: mu (K K^T)_aa,
+// the smallest term of the blocks) of the largest one's, all finite and far from the ends
+// of the range. Other cells keep doubles and BLOCK_FIX_NONE.
+template <class C, int D, int FORM>
+__device__ __forceinline__ void block_geometry_fixed(const SimtParams& p, long long e0, double* Gs, const double* Ws,
+                                                     double* Ks, int* Xs) {
+  constexpr bool CONV = FORM == FFC_NS_CONVECTION;
+  constexpr int PARTS = CONV ? C::NS : D * D;      // parts of a cell's blocks
+  constexpr int PLEN = CONV ? D : C::KRP;          // stored entries of a part
+  constexpr int PUSED = CONV ? D : D * D;          // entries used
+  const int t = threadIdx.x;
+  const int nc = int(p.n_elem - e0 < C::E ? p.n_elem - e0 : C::E);
+  int* Ts = Xs + C::E;      // [E] largest exponent of the blocks
+  int* Ls = Xs + 2 * C::E;  // [E] smallest exponent allowed for (convection: spread of the rows)
+  for (int el = t; el < nc; el += C::NT) {
+    double K[D][D], det;
+    bool degenerate, bad_index;
+    cell_geometry<D>(p.cells, p.vertices, p.n_vert, e0 + el, K, det, degenerate, bad_index);
+    if (degenerate) atomicOr(p.status, FFC_FLAG_DEGENERATE);
+    if (bad_index) atomicOr(p.status, FFC_FLAG_BOUNDS);
+    double* k = Ks + el * C::XD;
+    int lo = 1025, hi = -1022;
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+      int x = -1022;
+#pragma unroll
+      for (int b = 0; b < D; ++b) {
+        k[a * D + b] = K[a][b];
+        if constexpr (CONV) x = max(x, fix_exponent(K[a][b]));
+      }
+      if constexpr (!CONV) {
+#pragma unroll
+        for (int b = a; b < D; ++b) {
+          double s = 0.0;
+#pragma unroll
+          for (int c = 0; c < D; ++c) s = fma(K[a][c], K[b][c], s);
+          s *= det * p.mu;
+          k[D * D + 1 + sym_pair_index<D>(a, b)] = s;
+          if (a == b) x = fix_exponent(s);
+        }
+      }
+      lo = min(lo, x);
+      hi = max(hi, x);
+    }
+    k[D * D] = det;
+    Ts[el] = -1022;
+    Ls[el] = CONV ? hi - lo : lo;
+  }
+  __syncthreads();
+  for (int w = t; w < nc * PARTS; w += C::NT) {
+    const int el = w / PARTS, part = w - el * PARTS;
+    const double* K = Ks + el * C::XD;
+    const double det = K[D * D];
+    double* g = Gs + size_t(el) * C::NB * C::KRP + part * PLEN;
+    int top = -1022;
+    if constexpr (CONV) {
+      double wc[D];
+#pragma unroll
+      for (int c = 0; c < D; ++c) wc[c] = Ws[el * C::NCOEF + c * C::NS + part];
+#pragma unroll
+      for (int a = 0; a < D; ++a) {
+        double h = 0.0;
+#pragma unroll
+        for (int c = 0; c < D; ++c) h = fma(K[a * D + c], wc[c], h);
+        g[a] = det * h;
+        top = max(top, fix_exponent(g[a]));
+      }
+    } else {
+      const int c1 = part / D, c2 = part - c1 * D;
+      const double dm = det * p.mu, dl = det * p.lambda;
+#pragma unroll
+      for (int a1 = 0; a1 < D; ++a1) {
+        const double m1 = dm * K[a1 * D + c2], l1 = dl * K[a1 * D + c1];
+#pragma unroll
+        for (int a2 = 0; a2 < D; ++a2) {
+          const int ab = sym_pair_index<D>(a1 < a2 ? a1 : a2, a1 < a2 ? a2 : a1);
+          double v = c1 == c2 ? K[D * D + 1 + ab] : 0.0;
+          v = fma(l1, K[a2 * D + c2], fma(m1, K[a2 * D + c1], v));
+          g[a1 * D + a2] = v;
+          top = max(top, fix_exponent(v));
+        }
+      }
+    }
+    atomicMax(Ts + el, top);
+  }
+  __syncthreads();
+  for (int w = t; w < nc * PARTS; w += C::NT) {  // each thread its own parts again
+    const int el = w / PARTS, part = w - el * PARTS;
+    const int top = Ts[el], spread = CONV ? Ls[el] : top - Ls[el];
+    const bool fixed = top <= 900 && top >= -900 && spread <= (CONV ? 3 : 6);
+    if (part == 0) Xs[el] = fixed ? top * (1 << 20) : BLOCK_FIX_NONE;
+    if (!fixed) continue;
+    double* g = Gs + size_t(el) * C::NB * C::KRP + part * PLEN;
+    int2* gi = reinterpret_cast<int2*>(g);
+#pragma unroll
+    for (int k = 0; k < PUSED; ++k) gi[k] = fix_parts<C::BITS>(g[k], top);
   }
 }
 
@@ -160,6 +298,8 @@ __device__ __forceinline__ void block_tile(const SimtParams& p, long long tile, 
   T* Gs = reinterpret_cast<T*>(smem);                                       // [E][NB][KRP]
   const T* Rs = reinterpret_cast<const T*>(smem + C::G_BYTES);              // [NP2][KRP]
   double* Ws = reinterpret_cast<double*>(smem + C::G_BYTES + C::R_BYTES);   // [E][NCOEF]
+  double* Ks = reinterpret_cast<double*>(smem + C::G_BYTES + C::R_BYTES + C::W_BYTES);  // FP64: [E][XD]
+  int* Xs = reinterpret_cast<int*>(Ks + (C::FIX ? C::E * C::XD : 0));                    // FP64: [E] exponents
   const int t = threadIdx.x;
   const long long e0 = tile * C::E;
   if constexpr (C::NCOEF > 0) {
@@ -169,7 +309,8 @@ __device__ __forceinline__ void block_tile(const SimtParams& p, long long tile, 
   }
   __syncthreads();
   // ---- reduced geometry blocks of the tile's cells
-  for (int el = t; el < C::E; el += C::NT) {
+  if constexpr (C::FIX) block_geometry_fixed<C, D, FORM>(p, e0, Gs, Ws, Ks, Xs);
+  else for (int el = t; el < C::E; el += C::NT) {
     const long long e = e0 + el;
     T* g = Gs + size_t(el) * C::NB * C::KRP;
     // J^{-1} and det J in FP64 (measured: forming J^{-1} in FP32 from the FP64 adjugate,
@@ -235,39 +376,50 @@ __device__ __forceinline__ void block_tile(const SimtParams& p, long long tile, 
   }
   __syncthreads();
   // ---- contraction: the thread's slots x the group's cells
-  using V = typename std::conditional<sizeof(T) == 4, float4, double2>::type;
   constexpr bool DIAG = C::DIAG;
   constexpr int NPOS = DIAG ? D * D : D;  // element-tensor entries a slot writes per cell
   const int grp = C::NT >= C::NSL ? t / C::NSL : 0;
   const long long left = p.n_elem - e0;
   const int nc = int(left < C::E ? left : C::E);
-  // R[(s1,s2)] . block
-  auto contract = [&](const T* gblk, int j, const T* rrow) {
-    const V* gv = reinterpret_cast<const V*>(gblk);
-    T acc = T(0);
-#pragma unroll
-    for (int kv = 0; kv < C::KRP / C::VEC; ++kv) {
-      const V x = gv[kv];
-      T xs[C::VEC];
-      if constexpr (sizeof(T) == 4) {
-        xs[0] = x.x;
-        xs[1] = x.y;
-        xs[2] = x.z;
-        xs[3] = x.w;
-      } else {
-        xs[0] = x.x;
-        xs[1] = x.y;
+  // R[(s1,s2)] . block of cell el; `pipe`: FP64 results leave the fixed point on the FP64
+  // pipe (1) or on the integer ones (0)
+  auto contract = [&](const T* gblk, int el, int j, const T* rrow, int row, int pipe) {
+    if constexpr (C::FIX) {
+      const int eG = Xs[el];
+      if (eG == BLOCK_FIX_NONE) {
+        const double* R = static_cast<const double*>(p.a0) + size_t(row) * C::KR;
+        double acc = 0.0;
+        for (int k = 0; k < C::KR; ++k) acc = fma(gblk[k], __ldg(R + k), acc);
+        return acc;
       }
+      const int4* gv = reinterpret_cast<const int4*>(gblk);
+      FixAcc acc;
 #pragma unroll
-      for (int m = 0; m < C::VEC; ++m) {
-        const int k = kv * C::VEC + m;
-        if (k < C::KR) {
-          if constexpr (C::REG_R) acc = fma(xs[m], br.rr[j][k < C::KR ? k : 0], acc);
-          else acc = fma(xs[m], rrow[k], acc);
+      for (int k = 0; k < C::KR; k += 2) {
+        const int4 x = gv[k / 2];
+        acc.add(br.rr[j][k], make_int2(x.x, x.y));
+        if (k + 1 < C::KR) acc.add(br.rr[j][k + 1 < C::KR ? k + 1 : k], make_int2(x.z, x.w));
+      }
+      const int e20 = br.expo[j] + eG;
+      return pipe ? fix_to_double_fp64(acc.sum(), e20) : fix_to_double(acc.sum(), e20);
+    } else {
+      const float4* gv = reinterpret_cast<const float4*>(gblk);
+      T acc = T(0);
+#pragma unroll
+      for (int kv = 0; kv < C::KRP / C::VEC; ++kv) {
+        const float4 x = gv[kv];
+        const T xs[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+        for (int m = 0; m < C::VEC; ++m) {
+          const int k = kv * C::VEC + m;
+          if (k < C::KR) {
+            if constexpr (C::REG_R) acc = fma(xs[m], br.rr[j][k < C::KR ? k : 0], acc);
+            else acc = fma(xs[m], rrow[k], acc);
+          }
         }
       }
+      return acc;
     }
-    return acc;
   };
   using SG = BlockStaging<C, T, ASSEMBLE>;
   if constexpr (SG::ON) {
@@ -291,13 +443,13 @@ __device__ __forceinline__ void block_tile(const SimtParams& p, long long tile, 
           const T* gcell = Gs + size_t(el) * C::NB * C::KRP;
           T* cb = buf + size_t(el - c0) * C::NN;
           if constexpr (DIAG) {  // one value on the d diagonal positions
-            const T v = contract(gcell, j, rrow);
+            const T v = contract(gcell, el, j, rrow, s1 * C::NS + s2, 1);
 #pragma unroll
             for (int c = 0; c < D; ++c) cb[(c * C::NS + s1) * C::N + c * C::NS + s2] = v;
           } else {  // the row slot's d entries ((c1, s1), (c2, s2))
 #pragma unroll
             for (int c1 = 0; c1 < D; ++c1)
-              cb[(c1 * C::NS + s1) * C::N + c2 * C::NS + s2] = contract(gcell + (c1 * D + c2) * C::KRP, j, rrow);
+              cb[(c1 * C::NS + s1) * C::N + c2 * C::NS + s2] = contract(gcell + (c1 * D + c2) * C::KRP, el, j, rrow, s1 * C::NS + s2, 1);
           }
         }
       }
@@ -356,11 +508,11 @@ __device__ __forceinline__ void block_tile(const SimtParams& p, long long tile, 
         }
         const T* gcell = Gs + size_t(el) * C::NB * C::KRP;
         T vdiag = T(0);
-        if constexpr (DIAG) vdiag = contract(gcell, j, rrow);
+        if constexpr (DIAG) vdiag = contract(gcell, el, j, rrow, s1 * C::NS + s2, 1);
 #pragma unroll
         for (int m = 0; m < NPOS; ++m) {
           if (ASSEMBLE && !live_pos[m]) continue;
-          const T v = DIAG ? (live_pos[m] ? vdiag : T(0)) : contract(gcell + (m * D + c2) * C::KRP, j, rrow);
+          const T v = DIAG ? (live_pos[m] ? vdiag : T(0)) : contract(gcell + (m * D + c2) * C::KRP, el, j, rrow, s1 * C::NS + s2, m == 0);
           if constexpr (ASSEMBLE) {
             const int sv = sl[m];
             if (sv >= 0 && sv < p.nnz) atomicAdd(p.csr_val + sv, double(v));
