@@ -10,130 +10,248 @@
 // x_{c+1} - x_0, so dL/dx_{c+1} += dL/dJ[:, c] and dL/dx_0 -= sum_c dL/dJ[:, c]; the
 // vertex gradients are accumulated with FP64 atomic adds.
 //
-// One thread per cell. Only the symmetric part of Gbar enters (c = Gbar : K K^T with
-// K K^T symmetric, and Gbar + Gbar^T), so each thread accumulates the d(d+1)/2
-// combinations against the reference tensor in the kernels' symmetric layout (columns
-// (a,a) and (a,b) + (b,a)), held in shared memory and read as a broadcast (all lanes at
-// the same entry i); no cross-lane reductions. Then it runs the geometry chain rule
-// and scatters with atomics. FP64.
+// Only the symmetric part of Gbar enters, and A0 is symmetric in (i1, i2) (a symmetric
+// form, Section 3.5): with the d(d+1)/2 columns (a,a) and (a,b) + (b,a) of the kernels'
+// layout, gp[k] = sum_{i1 <= i2} A0[i1][i2][k] (dA[i1][i2] + dA[i2][i1]). That contraction
+// runs in fixed point (fixed_point.cuh): in FP64 its n^2 d(d+1)/2 multiply-adds held the
+// FP64 pipe at 95% (P2 tetrahedra: 300 of the 381 SM clocks a cell took).
+//
+// Every warp works by itself (no CTA barrier after the start, so the load, integer and FP64
+// phases of different warps overlap) on tiles of up to 32 cells:
+//   load         the dA of 32/L cells at a time, asynchronously into shared memory, rows
+//                padded to an odd number of doubles;
+//   contraction  L lanes per cell: the cell's largest exponent first, then each pair i1 <= i2
+//                rounded to 55-57 bits, its two halves added as integers, times the
+//                fixed-point A0 of the pair; the L partial sums are added as integers;
+//   chain rule   one lane per cell of the tile: FP64 J^-1, |det J| and the formula above, and
+//                FP64 atomics to the d+1 vertices.
+// Bound by the FP64 geometry and chain rule (pipe 49% busy) and the integer instructions
+// (issue 44%) at 20 resident warps. Backward pass, FP64 multiply-adds -> here: P2 on 1.05 M
+// tetrahedra 1390 -> 490 us (730-890 us with CTA-wide phases and a barrier between them),
+// P3 on 82,944 628 -> 166, P4 on 24,576 580 -> 181, P1 on 663,552 340 -> 220 us.
+// A cell whose dA is not finite or lies outside [2^-900, 2^900] takes FP64 multiply-adds
+// over all n^2 entries instead, so infinities and NaN reach the same gradients as there.
 #include <cuda_runtime.h>
 
 #include "ffc_internal.h"
+#include "fixed_point.cuh"
 #include "geometry.cuh"
 
 namespace ffc {
 namespace {
 
-constexpr int THREADS = 256;
-
 template <int D, int Q>
-__global__ void __launch_bounds__(THREADS) poisson_adjoint_kernel(const int32_t* __restrict__ cells,
-                                                                 const double* __restrict__ vertices,
-                                                                 long long n_vert, const double* __restrict__ a0t,
-                                                                 const double* __restrict__ dA, double* dvert,
-                                                                 long long n_elem, unsigned* status) {
-  constexpr int N = nscalar(D, Q);
-  constexpr int NN = N * N;
-  constexpr int NP = D * (D + 1) / 2;
-  // the reference tensor in the symmetric layout, one row per entry i:
-  // P[i][aa] = A0[i][(a,a)], P[i][ab] = A0[i][(a,b)] + A0[i][(b,a)] (a < b)
-  extern __shared__ double a0s[];  // [NN][NP]
-  for (int k = threadIdx.x; k < NN * NP; k += blockDim.x) {
-    const int i = k / NP, pidx = k % NP;
-    a0s[k] = a0t[pidx * NN + i];
-  }
-  __syncthreads();
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n_elem;
-       e += (long long)gridDim.x * blockDim.x) {
-    // gp[aa] = Gbar[a][a], gp[ab] = Gbar[a][b] + Gbar[b][a]
-    double gp[NP];
+struct AdjCfg {
+  static constexpr int N = nscalar(D, Q);
+  static constexpr int NN = N * N;
+  static constexpr int NP = D * (D + 1) / 2;
+  static constexpr int NE = N * (N + 1) / 2;
+  // lanes per cell: 4-10 KB of staged dA per warp
+  static constexpr int L = NN <= 16 ? 1 : (NN <= 64 ? 2 : (NN <= 128 ? 4 : (NN <= 256 ? 8 : (NN <= 512 ? 16 : 32))));
+  static constexpr int CW = 32 / L;      // cells of a batch
+  static constexpr int STRIDE = NN | 1;  // doubles of a staged row: odd, no bank conflicts over cells
+  // warps per CTA: 16 in one CTA where the reference tensor takes 30 KB (P4 tetrahedra)
+  static constexpr int WARPS = NE * NP > 2000 ? 16 : 4;
+  static constexpr int MIN_BLOCKS = WARPS > 4 ? 1 : 6;
+  // bits of a factor: NE products of high parts h <= 2^(BITS - 29) are summed in 63 bits
+  static constexpr int BITS = NE > 217 ? 55 : (NE > 100 ? 56 : 57);
+  static_assert(double(NE) * double(1ull << (2 * (BITS - 29))) < 9.0e18, "the sums must fit in 63 bits");
+  static constexpr int ROWS = CW * STRIDE;  // doubles of a warp's staged rows
+  static constexpr int WBUF = ROWS + 32 * NP;  // and its cells' sums
+  static constexpr size_t SMEM = size_t(WARPS) * WBUF * 8 + size_t(NE) * NP * 8 + size_t(NE) * 4 + size_t(NP) * 4;
+};
+
+// the geometry chain rule of one cell and its atomics; S = Gbar + Gbar^T
+//   dL/dJ = s (c I - P) K^T,  P = K^T S K,  c = tr(P) / 2
+// (the formula above with K taken out on the right: 90 FP64 operations instead of 120)
+template <int D>
+__device__ __forceinline__ void adjoint_chain(const double K[D][D], double s, const double S[D][D], const int* id,
+                                              double* dvert) {
+  double W[D][D], P[D][D], c = 0.0;
 #pragma unroll
-    for (int k = 0; k < NP; ++k) gp[k] = 0.0;
-    const double* row = dA + e * NN;
-#pragma unroll 4
-    for (int i = 0; i < NN; ++i) {
-      const double g = __ldg(row + i);
-#pragma unroll
-      for (int k = 0; k < NP; ++k) gp[k] = fma(a0s[i * NP + k], g, gp[k]);
-    }
-    double K[D][D], s;
-    bool degenerate, bad_index;
-    cell_geometry<D>(cells, vertices, n_vert, e, K, s, degenerate, bad_index);
-    if (degenerate) atomicOr(status, FFC_FLAG_DEGENERATE);
-    if (bad_index) {
-      atomicOr(status, FFC_FLAG_BOUNDS);
-      continue;
-    }
-    double M[D][D];  // K K^T
-#pragma unroll
-    for (int a = 0; a < D; ++a)
-#pragma unroll
-      for (int b = 0; b < D; ++b) {
-        double t = 0.0;
-#pragma unroll
-        for (int k = 0; k < D; ++k) t += K[a][k] * K[b][k];
-        M[a][b] = t;
-      }
-    // S = Gbar + Gbar^T, c = Gbar : M (M symmetric)
-    double S[D][D], c = 0.0;
-#pragma unroll
-    for (int a = 0; a < D; ++a)
-#pragma unroll
-      for (int b = 0; b < D; ++b) {
-        const double v = gp[sym_pair_index<D>(a < b ? a : b, a < b ? b : a)];
-        S[a][b] = (a == b) ? 2.0 * v : v;
-        if (a <= b) c += v * M[a][b];
-      }
-    // T = S M ; dJ = s (c K^T - K^T T)
-    double T[D][D];
-#pragma unroll
-    for (int a = 0; a < D; ++a)
-#pragma unroll
-      for (int b = 0; b < D; ++b) {
-        double t = 0.0;
-#pragma unroll
-        for (int k = 0; k < D; ++k) t += S[a][k] * M[k][b];
-        T[a][b] = t;
-      }
-    double dJ[D][D];
-#pragma unroll
-    for (int r = 0; r < D; ++r)
-#pragma unroll
-      for (int col = 0; col < D; ++col) {
-        double t = 0.0;
-#pragma unroll
-        for (int k = 0; k < D; ++k) t += K[k][r] * T[k][col];
-        dJ[r][col] = s * (c * K[col][r] - t);
-      }
-    int id[D + 1];
-#pragma unroll
-    for (int j = 0; j <= D; ++j) id[j] = __ldg(cells + e * (D + 1) + j);
+  for (int a = 0; a < D; ++a)
 #pragma unroll
     for (int r = 0; r < D; ++r) {
-      double sum = 0.0;
+      double t = 0.0;
 #pragma unroll
-      for (int col = 0; col < D; ++col) {
-        atomicAdd(dvert + (long long)id[col + 1] * D + r, dJ[r][col]);
-        sum += dJ[r][col];
-      }
-      atomicAdd(dvert + (long long)id[0] * D + r, -sum);
+      for (int b = 0; b < D; ++b) t = fma(S[a][b], K[b][r], t);
+      W[a][r] = t;
     }
+#pragma unroll
+  for (int r = 0; r < D; ++r)
+#pragma unroll
+    for (int m = r; m < D; ++m) {
+      double t = 0.0;
+#pragma unroll
+      for (int a = 0; a < D; ++a) t = fma(K[a][r], W[a][m], t);
+      P[r][m] = P[m][r] = t;
+    }
+#pragma unroll
+  for (int r = 0; r < D; ++r) c += P[r][r];
+  c *= 0.5 * s;
+  double Qm[D][D];
+#pragma unroll
+  for (int r = 0; r < D; ++r)
+#pragma unroll
+    for (int m = r; m < D; ++m) Qm[r][m] = Qm[m][r] = r == m ? fma(-s, P[r][r], c) : -s * P[r][m];
+#pragma unroll
+  for (int r = 0; r < D; ++r) {
+    double sum = 0.0;
+#pragma unroll
+    for (int col = 0; col < D; ++col) {
+      double t = 0.0;
+#pragma unroll
+      for (int m = 0; m < D; ++m) t = fma(Qm[r][m], K[col][m], t);
+      atomicAdd(dvert + (long long)id[col + 1] * D + r, t);
+      sum += t;
+    }
+    atomicAdd(dvert + (long long)id[0] * D + r, -sum);
+  }
+}
+
+__device__ __forceinline__ void adj_copy8(double* dst, const double* src) {
+  const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(dst));
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(src) : "memory");
+}
+
+// `tile_cells`: cells of a warp's tile, a multiple of CW, at most 32
+template <int D, int Q>
+__global__ void __launch_bounds__(AdjCfg<D, Q>::WARPS * 32, AdjCfg<D, Q>::MIN_BLOCKS)
+    poisson_adjoint_kernel(const int32_t* __restrict__ cells, const double* __restrict__ vertices, long long n_vert,
+                           const double* __restrict__ a0t, const double* __restrict__ dA, double* dvert,
+                           long long n_elem, int tile_cells, unsigned* status) {
+  using C = AdjCfg<D, Q>;
+  constexpr int N = C::N, NN = C::NN, NP = C::NP, NE = C::NE, L = C::L, NT = C::WARPS * 32;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  int2* as = reinterpret_cast<int2*>(smem_raw);                      // [NE][NP] A0, fixed point
+  double* wbuf = reinterpret_cast<double*>(as + NE * NP);            // [WARPS][WBUF]
+  unsigned* pairs = reinterpret_cast<unsigned*>(wbuf + C::WARPS * C::WBUF);  // [NE] positions of (i1, i2), (i2, i1)
+  int* ae = reinterpret_cast<int*>(pairs + NE);                      // [NP] exponents of A0's columns
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  if (t < NP) ae[t] = -1022;
+  for (int u = t; u < NE; u += NT) {
+    int i1 = 0, v = u;
+    while (v >= N - i1) v -= N - i1++;  // row i1 holds the pairs (i1, i1 .. N-1)
+    pairs[u] = unsigned(i1 * N + i1 + v) | (unsigned((i1 + v) * N + i1) << 16);
+  }
+  __syncthreads();
+  for (int w = t; w < NE * NP; w += NT)
+    atomicMax(ae + w % NP, fix_exponent(__ldg(a0t + (w % NP) * NN + (pairs[w / NP] & 0xffffu))));
+  __syncthreads();
+  for (int w = t; w < NE * NP; w += NT)
+    as[w] = fix_parts<C::BITS>(__ldg(a0t + (w % NP) * NN + (pairs[w / NP] & 0xffffu)), ae[w % NP]);
+  __syncthreads();
+  double* rows = wbuf + warp * C::WBUF;  // [CW][STRIDE] dA of the batch
+  double* gp = rows + C::ROWS;           // [32][NP] Gbar + Gbar^T of the tile's cells
+  const int bc = lane / L, l = lane % L;
+  const unsigned mask = L == 32 ? 0xffffffffu : ((1u << (L % 32)) - 1u) << (bc * L);
+  const long long n_tiles = (n_elem + tile_cells - 1) / tile_cells;
+  for (long long tile = (long long)blockIdx.x * C::WARPS + warp; tile < n_tiles;
+       tile += (long long)gridDim.x * C::WARPS) {
+    const long long e0 = tile * tile_cells;
+    const int nc = int(n_elem - e0 < tile_cells ? n_elem - e0 : tile_cells);
+    for (int b = 0; b < nc; b += C::CW) {
+      const int nb = min(C::CW, nc - b);
+      if (bc < nb) {  // each cell's lanes copy its row: 8 L contiguous bytes a row and step
+        const double* src = dA + (e0 + b + bc) * NN;
+#pragma unroll 5
+        for (int k = l; k < NN; k += L) adj_copy8(rows + bc * C::STRIDE + k, src + k);
+      }
+      asm volatile("cp.async.wait_all;\n" ::: "memory");
+      __syncwarp();
+      if (bc < nb) {
+        const double* x = rows + bc * C::STRIDE;
+        int top = -1022;
+#pragma unroll 5
+        for (int k = l; k < NN; k += L) top = max(top, fix_exponent(x[k]));
+#pragma unroll
+        for (int o = L / 2; o > 0; o >>= 1) top = max(top, __shfl_xor_sync(mask, top, o));
+        bool fixed = top <= 900 && top >= -900;
+        if (top == -1022) {  // all zero (the gradients of local functionals mostly are) or denormal
+          int any = 0;
+          for (int k = l; k < NN; k += L) any |= x[k] != 0.0;
+#pragma unroll
+          for (int o = L / 2; o > 0; o >>= 1) any |= __shfl_xor_sync(mask, any, o);
+          fixed = any == 0;
+        }
+        if (fixed) {
+          FixAcc acc[NP];
+#pragma unroll 2
+          for (int u = l; u < NE; u += L) {
+            const unsigned pq = pairs[u];
+            const int p1 = int(pq & 0xffffu), p2 = int(pq >> 16);
+            long long f = fix_round<C::BITS>(x[p1], top + 1);
+            if (p1 != p2) f += fix_round<C::BITS>(x[p2], top + 1);
+            const int2 g = fix_split(f);
+            const int2* a = as + u * NP;
+#pragma unroll
+            for (int k = 0; k < NP; ++k) acc[k].add(a[k], g);
+          }
+#pragma unroll
+          for (int k = 0; k < NP; ++k) {
+            long long v = acc[k].sum();
+#pragma unroll
+            for (int o = L / 2; o > 0; o >>= 1) v += __shfl_xor_sync(mask, v, o);
+            // a diagonal entry of Gbar + Gbar^T is twice Gbar's
+            if (l == 0)
+              gp[(b + bc) * NP + k] =
+                  fix_to_double(v, (ae[k] + top + 1 + 58 - 2 * C::BITS + (k < D ? 1 : 0)) * (1 << 20));
+          }
+        } else if (l == 0) {
+          double g[NP];
+#pragma unroll
+          for (int k = 0; k < NP; ++k) g[k] = 0.0;
+          for (int i = 0; i < NN; ++i) {
+#pragma unroll
+            for (int k = 0; k < NP; ++k) g[k] = fma(__ldg(a0t + k * NN + i), x[i], g[k]);
+          }
+#pragma unroll
+          for (int k = 0; k < NP; ++k) gp[(b + bc) * NP + k] = k < D ? 2.0 * g[k] : g[k];
+        }
+      }
+      __syncwarp();  // the rows are overwritten next; the sums are read below
+    }
+    if (lane < nc) {
+      const long long e = e0 + lane;
+      double K[D][D], s, S[D][D];
+      bool degenerate, bad_index;
+      cell_geometry<D>(cells, vertices, n_vert, e, K, s, degenerate, bad_index);
+      if (degenerate) atomicOr(status, FFC_FLAG_DEGENERATE);
+      if (bad_index) {
+        atomicOr(status, FFC_FLAG_BOUNDS);
+      } else {
+#pragma unroll
+        for (int a = 0; a < D; ++a)
+#pragma unroll
+          for (int b = 0; b < D; ++b) S[a][b] = gp[lane * NP + sym_pair_index<D>(a < b ? a : b, a < b ? b : a)];
+        int id[D + 1];
+#pragma unroll
+        for (int j = 0; j <= D; ++j) id[j] = __ldg(cells + e * (D + 1) + j);
+        adjoint_chain<D>(K, s, S, id, dvert);
+      }
+    }
+    __syncwarp();  // the next tile's sums overwrite gp
   }
 }
 
 template <int D, int Q>
 int run(const LaunchArgs& a, const double* dA, double* dvert) {
-  constexpr int N = nscalar(D, Q);
-  constexpr size_t SMEM = size_t(D * (D + 1) / 2) * N * N * sizeof(double);
+  using C = AdjCfg<D, Q>;
   auto kern = poisson_adjoint_kernel<D, Q>;
+  constexpr int NT = C::WARPS * 32;
   int sms = 0, per_sm = 1;
-  if (launch_config(reinterpret_cast<const void*>(kern), THREADS, SMEM, -1, &sms, &per_sm) != FFC_OK)
+  if (launch_config(reinterpret_cast<const void*>(kern), NT, C::SMEM, 100, &sms, &per_sm) != FFC_OK)
     return FFC_ECUDA;
+  // tiles of 32 cells keep every lane in the chain rule; meshes of fewer cells than that per
+  // resident warp take fewer (whole batches), so that the batches spread over the warps
+  const long long warps = (long long)sms * per_sm * C::WARPS;
+  long long tile = (a.n_elem + warps - 1) / warps;
+  tile = tile >= 32 ? 32 : (tile + C::CW - 1) / C::CW * C::CW;
   long long grid = (long long)sms * per_sm;
-  const long long need = (a.n_elem + THREADS - 1) / THREADS;
+  const long long need = (a.n_elem + tile * C::WARPS - 1) / (tile * C::WARPS);
   if (grid > need) grid = need;
-  kern<<<unsigned(grid), THREADS, SMEM, static_cast<cudaStream_t>(a.stream)>>>(
-      a.cells, a.vertices, a.n_vert, a.t->a0t_f64, dA, dvert, a.n_elem, a.status);
+  kern<<<unsigned(grid), NT, C::SMEM, static_cast<cudaStream_t>(a.stream)>>>(
+      a.cells, a.vertices, a.n_vert, a.t->a0t_f64, dA, dvert, a.n_elem, int(tile), a.status);
   return cudaPeekAtLastError() == cudaSuccess ? FFC_OK : FFC_ECUDA;
 }
 

@@ -27,18 +27,18 @@ __device__ __forceinline__ int fix_exponent(double x) {
   return int((unsigned(__double2hiint(x)) >> 20) & 0x7ffu) - 1022;
 }
 
-// x 2^(B - e) rounded to the nearest integer (halves away from zero), |x| < 2^e
+// x 2^(B - e) rounded to the nearest integer (halves away from zero), |x| < 2^e, 52 <= B <= 59
 template <int B>
 __device__ __forceinline__ long long fix_round(double x, int e) {
-  const unsigned hw = unsigned(__double2hiint(x));
-  const int ex = int((hw >> 20) & 0x7ffu);
-  unsigned long long m = (static_cast<unsigned long long>(hw & 0xfffffu) << 32) | unsigned(__double2loint(x));
-  if (ex) m |= 1ull << 52;
-  const int sh = (ex ? ex : 1) - 1075 + B - e;  // x = +-m 2^(ex - 1075)
-  unsigned long long f;
-  if (sh >= 0) f = m << (sh < 63 ? sh : 63);
-  else f = -sh < 64 ? (m + (1ull << (-sh - 1))) >> -sh : 0ull;
-  return (hw >> 31) ? -static_cast<long long>(f) : static_cast<long long>(f);
+  static_assert(B >= 52 && B <= 59, "the significand is shifted left by B - 52, then right");
+  const int hw = __double2hiint(x);
+  const int ex = int((unsigned(hw) >> 20) & 0x7ffu);
+  const unsigned mh = (unsigned(hw) & 0xfffffu) | (ex ? 1u << 20 : 0u);
+  const unsigned long long m = (static_cast<unsigned long long>(mh) << 32 | unsigned(__double2loint(x))) << (B - 52);
+  const int sh = e + 1022 - (ex ? ex : 1);  // >= 0
+  const long long f = static_cast<long long>(((m >> (sh < 63 ? sh : 63)) + 1) >> 1);
+  const long long s = hw >> 31;
+  return (f ^ s) - s;
 }
 
 // The two parts (h, l) of a fixed-point factor. The empty asm hides that they came from a

@@ -90,9 +90,10 @@ struct BlockCfg {
   static constexpr size_t SMEM = G_BYTES + R_BYTES + W_BYTES + X_BYTES;
   // register budget of the single-form FP32 kernel: two resident CTAs of 257..511 threads
   // (up to 78 registers), three of up to 256; FP64 keeps its reduced rows in registers
-  // without spills (a bound for two CTAs: elasticity P3 1262 against 945 us; for three:
-  // convection P2 986 against 816 us)
-  static constexpr int MIN_BLOCKS = sizeof(T) == 8 ? 1 : (NT >= 512 ? 1 : (NT > 256 ? 2 : 3));
+  // without spills: two CTAs of up to 256 threads (convection P2 with one: 1122 against
+  // 810 us, with three and spills 986 us), one of more (elasticity P3 with two: 1262
+  // against 945 us)
+  static constexpr int MIN_BLOCKS = sizeof(T) == 8 ? (NT <= 256 ? 2 : 1) : (NT >= 512 ? 1 : (NT > 256 ? 2 : 3));
 };
 
 template <class C, typename T>
