@@ -298,7 +298,7 @@ void ffc_batch_destroy(ffc_batch* b);
  *   row_ptr  device int64 [n_dof + 1], col device int32 [nnz]: the pattern of
  *            ffc_csr_pattern (columns sorted within each row), copied to the device
  * The plan stores, per chunk, the chunk's pairs grouped by local index i1 as
- * e * n_local + i1, the work units (pieces of one group), and for every pair and local
+ * e * n_local + i1, the groups' extents, and for every pair and local
  * column i2 the position of column dofmap[e][i2] inside the chunk (uint16). It owns
  * about n_elem * n_local * (2 * n_local + 4) + n_dof * 8 bytes of device memory plus an
  * [n_elem][12]-double geometry scratch (ffc_row_plan_layout reports the exact figure);
@@ -314,7 +314,7 @@ int ffc_row_plan_create(int64_t n_elem, int n_local, const int32_t* dofmap, int6
 /* Rows, stored entries, longest row and most cells sharing one dof. */
 int ffc_row_plan_info(const ffc_row_plan* p, int64_t* n_dof, int64_t* nnz, int* max_row, int* max_incidence);
 /* Chunks, entries and pairs of the largest chunk, bytes of the largest chunk's plan data
- * (work units, pairs and positions) and the plan's device memory in bytes. Any output
+ * (group extents, pairs and positions) and the plan's device memory in bytes. Any output
  * pointer may be NULL. */
 int ffc_row_plan_layout(const ffc_row_plan* p, int64_t* n_chunks, int* max_chunk_values, int* max_chunk_pairs,
                         int* max_region_bytes, int64_t* device_bytes);
@@ -327,7 +327,8 @@ void ffc_row_plan_destroy(ffc_row_plan* p);
  * for every k < nnz (overwritten). cells / vertices / n_vert as for ffc_tabulate, for
  * the cells the plan was built from. precision FFC_FP32: G_K and the contraction in
  * FP32 exactly as ffc_assemble computes them (the same contributions), FFC_FP64: in FP64.
- * Two launches on `stream`: the geometry tensors into the plan's scratch, then the rows.
+ * Three launches on `stream`: the geometry tensors and the chunks' bounds into the plan's
+ * scratch, then the rows.
  * Calls that share a plan must be ordered on one stream (they share the scratch).
  * A non-finite G_K (a degenerate cell, FFC_FLAG_DEGENERATE) makes the values of the
  * chunk that holds its rows NaN. Other forms: FFC_EUNSUPPORTED. The plan's n_local must

@@ -28,7 +28,7 @@
 // Bound by the FP64 geometry and chain rule (pipe 49% busy) and the integer instructions
 // (issue 44%) at 20 resident warps. Backward pass, FP64 multiply-adds -> here: P2 on 1.05 M
 // tetrahedra 1390 -> 490 us (730-890 us with CTA-wide phases and a barrier between them),
-// P3 on 82,944 628 -> 166, P4 on 24,576 580 -> 181, P1 on 663,552 340 -> 220 us.
+// P3 on 82,944 501 -> 166, P4 on 24,576 586 -> 181, P1 on 663,552 320 -> 220 us.
 // A cell whose dA is not finite or lies outside [2^-900, 2^900] takes FP64 multiply-adds
 // over all n^2 entries instead, so infinities and NaN reach the same gradients as there.
 #include <cuda_runtime.h>

@@ -2,7 +2,9 @@
 // tensor, the library-owned status word, and dispatch to the kernels.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <climits>
+#include <cmath>
 #include <map>
 #include <cstring>
 #include <mutex>
@@ -134,7 +136,22 @@ int ensure_device_tensors(ffc_form* f, DeviceTensors** out) {
       for (size_t a = 0; a < na; ++a)
         for (size_t i2 = 0; i2 < n; ++i2) soa[(i1 * na + a) * n + i2] = rows[(i1 * n + i2) * na + a];
     std::vector<float> soa32(soa.begin(), soa.end());
-    if ((rc = upload(&t.a0s_f64, soa)) || (rc = upload(&t.a0s_f32, soa32))) {
+    std::vector<double> most(n, 0.0);
+    std::vector<float> most32(n, 0.f);
+    for (size_t i1 = 0; i1 < n; ++i1)
+      for (size_t k = i1 * n * na; k < (i1 + 1) * n * na; ++k) {
+        most[i1] = std::max(most[i1], std::fabs(soa[k]));
+        most32[i1] = std::max(most32[i1], std::fabs(soa32[k]));
+      }
+    const size_t nap = (na + 3) / 4 * 4;
+    std::vector<float> padded;
+    if (f->kind == FFC_POISSON) {
+      padded.assign(nn * nap, 0.f);
+      for (size_t i = 0; i < nn; ++i)
+        for (size_t a = 0; a < na; ++a) padded[i * nap + a] = rows32[i * na + a];
+    }
+    if ((!padded.empty() && (rc = upload(&t.a0v_f32, padded))) || (rc = upload(&t.a0s_f64, soa)) || (rc = upload(&t.a0s_f32, soa32)) || (rc = upload(&t.a0m_f64, most)) ||
+        (rc = upload(&t.a0m_f32, most32))) {
       cudaFree(t.a0_f64);
       cudaFree(t.a0t_f64);
       cudaFree(t.a0_f32);
@@ -143,6 +160,9 @@ int ensure_device_tensors(ffc_form* f, DeviceTensors** out) {
       cudaFree(t.r_f32);
       cudaFree(t.a0s_f64);
       cudaFree(t.a0s_f32);
+      cudaFree(t.a0v_f32);
+      cudaFree(t.a0m_f64);
+      cudaFree(t.a0m_f32);
       return rc;
     }
   }
@@ -168,6 +188,9 @@ void release_device_tensors(ffc_form* f) {
     cudaFree(t.r_f32);
     cudaFree(t.a0s_f64);
     cudaFree(t.a0s_f32);
+    cudaFree(t.a0v_f32);
+    cudaFree(t.a0m_f64);
+    cudaFree(t.a0m_f32);
   }
   f->dev.clear();
   cudaSetDevice(cur);

@@ -22,6 +22,11 @@ struct DeviceTensors {
   // whose lanes take consecutive columns i2 of one row i1)
   double* a0s_f64 = nullptr;
   float* a0s_f32 = nullptr;
+  // Poisson: [n][n][na padded to a multiple of 4] (the FP32 row-owner kernels' vector loads)
+  float* a0v_f32 = nullptr;
+  // and the largest magnitude of each row i1 ([n]; the row-owner kernels' bounds)
+  double* a0m_f64 = nullptr;
+  float* a0m_f32 = nullptr;
   // tcgen05 operands: A0 split into TF32 (family 0: 2 parts) or BF16 (family 1: 3 parts),
   // each part laid out per 128-entry M-tile in the core-matrix layout
   void* tc_part[2][3] = {{nullptr, nullptr, nullptr}, {nullptr, nullptr, nullptr}};

@@ -12,17 +12,23 @@
 // zeroing pass, every value written exactly once.
 //
 // Work layout inside a chunk. The plan stores each chunk's pairs grouped by local index
-// i1 (a "class"; within a class the pairs of different rows alternate), the work units
-// (pieces of a class), and per pair the chunk-relative positions of its columns i2 =
-// 0..n-1. A warp takes one unit: the reference-tensor entries A0[i1][i2][.] its lanes
-// need stay in registers for the whole unit, each pair's G_K is a shared-memory
-// broadcast, and one warp instruction adds the contributions of one element-tensor row
-// (or of a few rows of different global rows), whose positions are distinct: the
-// shared-memory atomics meet no same-address conflicts and few bank conflicts. For n
-// >= 32 lane l takes column l of every pair (and the columns beyond 32 are spread over the
-// lanes); for n < 32 the unit's (pair, column) items are spread over the lanes in order.
-// Later chunks' plan data and geometry tensors are staged in shared memory with cp.async
-// while the current chunk is summed and the previous one written out.
+// i1 (a "class"; within a class the pairs of different rows alternate), the class runs, the
+// run in which each of 32 equal shares of the pairs begins, and per pair the chunk-relative
+// positions of its columns i2 = 0..n-1. Every warp sums one share: the reference-tensor
+// entries A0[i1][i2][.] its lanes need stay in registers for a class run, each pair's G_K is
+// a shared-memory broadcast, and one warp instruction adds the contributions of one
+// element-tensor row (or of a few rows of different global rows), whose positions are
+// distinct: the shared-memory atomics meet no same-address conflicts and few bank conflicts.
+// For n >= 32 lane l takes column l of every pair (and the columns beyond 32 are packed over
+// the lanes of separate steps); for n < 32 a warp takes 32 / n pairs side by side. Later
+// chunks' plan data and geometry tensors are staged in shared memory with cp.async while the
+// current chunk is summed and the previous one written out.
+//
+// What bounds it: the L1 / shared-memory data pipe (71% busy for P4: bank conflicts of the
+// atomics, 2.7 cycles each, plan copies, write-out) and instruction issue (65%). Measured,
+// a queue of warp tasks with in-loop bounds and 64-bit conversions -> equal shares: mass +
+// Poisson pair, P3 on 215,622 tets 496 -> 354 us, P4 on 663,552 tets 3493 -> 2953 us (0.43
+// of HBM on 8.68 GB), P2 on 384,000 tets 347 -> 252 us, P4 on 180,000 triangles 564 -> 184 us.
 //
 // Fixed-point accumulation. The sums are kept in fixed point with one unit per chunk and
 // form, where 2^(eb-1) bounds every partial sum of every entry of the chunk (the largest
@@ -36,9 +42,8 @@
 // 32-bit shared atomics run about seven times faster than 64-bit ones on this GPU.
 // Chunks whose bound lies outside the range of the FP32 scale, and FP64 contributions,
 // take an integer conversion instead (truncation, error < u). The value of an entry is
-// the digit sums' value in units u, rounded once to FP64 in integer arithmetic (the FP64
-// pipe's integer conversion takes half of them where it is exact). Integer addition is
-// exact and associative, so the result does not depend on the order of the additions:
+// the digit sums' value in units u, rounded once to FP64 in integer arithmetic. Integer
+// addition is exact and associative, so the result does not depend on the order of the additions:
 // per entry |result - exact sum of the contributions| <= m u / 2 + an ulp of the result
 // (m contributions; u / 2 < 2^-30 B for FP32, 2^-61 B for FP64, B the chunk's bound), and
 // the matrix is reproducible bit for bit.
@@ -49,6 +54,7 @@
 #include <climits>
 #include <cstring>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "ffc_internal.h"
@@ -59,32 +65,22 @@ namespace {
 
 constexpr int ROWS_VMAX = 4096;           // values of one chunk (shared-memory accumulators)
 constexpr int ROWS_VSTRIDE = ROWS_VMAX + 4;  // ints of one digit array: a chunk's values, shifted by 0 or 1
-constexpr int ROWS_PMAX = 320;            // pairs of one chunk
+constexpr int ROWS_PMAX = 320;            // pairs of one chunk (a multiple of 32)
 constexpr int ROWS_MAX_INCIDENCE = 1023;  // digit sums of 21-bit digits stay within 32 bits
 constexpr int ROWS_MAX_LOCAL = 64;        // local dofs per cell the plan carries
 
-// Pairs of one work unit: a warp takes the pairs of one class i1 in pieces of at most this
-// many (larger pieces for small element tensors, whose units hold several pairs per step;
-// short ones where a lane takes a column of a pair, so that an iteration's tasks are many
-// and short and its warps finish together).
-#ifndef ROWS_UMAX_WIDE
-#define ROWS_UMAX_WIDE 16
-#endif
-__host__ __device__ constexpr int rows_umax(int n) { return n <= 6 ? 32 : (n < 32 ? 16 : ROWS_UMAX_WIDE); }
-// Work units a chunk of P pairs can have: every non-empty class gives ceil(m / umax) <=
-// m / umax + 1 pieces.
-__host__ __device__ constexpr int region_unit_slots(int n, long long P) {
-  return int((n < P ? n : P) + P / rows_umax(n));
-}
+constexpr int ROWS_WARPS = 32;            // equal shares of a chunk's pairs the plan prepares
+
+// Class runs of a chunk of P pairs: at most one per local index i1.
+__host__ __device__ constexpr int region_runs(int n, long long P) { return int(n < P ? n : P); }
 
 // A chunk's region of plan data (16-byte aligned, a multiple of 16 bytes):
-//   uint32 n_units
-//   uint32 unit[region_unit_slots(n, P)]  work units i1 | k0 << 7 | k1 << 19: pairs
-//                                        [k0, k1) of class i1, in class order
-//   int32  pr[P]       the pairs e * n + i1, grouped by class
-//   uint16 pos[P][n]   chunk-relative value index of column i2 of each pair
+//   uint8  first[ROWS_WARPS]  the run that holds pair P w / ROWS_WARPS, the first of share w
+//   uint32 run[region_runs]   i1 | k0 << 7 | k1 << 19: pairs [k0, k1) are class i1, in order
+//   int32  pr[P]              the pairs e * n + i1, grouped by class
+//   uint16 pos[P][n]          chunk-relative value index of column i2 of each pair
 __host__ __device__ constexpr long long region_pr_offset(int n, long long P) {
-  return 4ll * (1 + region_unit_slots(n, P));
+  return ROWS_WARPS + 4ll * region_runs(n, P);
 }
 __host__ __device__ constexpr long long region_bytes(int n, long long P) {
   return (region_pr_offset(n, P) + 4 * P + 2 * P * n + 15) / 16 * 16;
@@ -114,6 +110,7 @@ struct ffc_row_plan {
   int32_t* chunk_inc = nullptr;     // [n_chunks] most pairs of one row in the chunk
   unsigned char* region = nullptr;  // [region_total] chunk regions (see region_bytes)
   void* geom = nullptr;             // per-cell geometry scratch, [n_elem][12] doubles
+  int2* chunk_eb = nullptr;         // [n_chunks] scratch: the chunk's bound exponents (two forms)
 };
 
 namespace ffc {
@@ -230,8 +227,8 @@ __global__ void plan_fill(const int32_t* __restrict__ dofmap, long long total, l
 // One thread per chunk: the chunk's pairs grouped by class i1; within a class ordered by
 // (rank of the pair among the class's pairs of its row, row, cell), so consecutive pairs
 // of a class belong to different rows where the class has several. Writes the ordered
-// pairs and the work units (each class cut into pieces of at most rows_umax(n) pairs)
-// into the chunk's region. `key` is scratch [total].
+// pairs, the class runs and the first run of each share into the chunk's region. `key` is
+// scratch [total].
 __global__ void plan_sort(const int32_t* __restrict__ dofmap, const int32_t* __restrict__ chunk_row,
                           const int32_t* __restrict__ chunk_pair, const int64_t* __restrict__ chunk_off,
                           long long n_chunks, int n, const int32_t* __restrict__ inc_tmp,
@@ -242,7 +239,7 @@ __global__ void plan_sort(const int32_t* __restrict__ dofmap, const int32_t* __r
     const int r0 = chunk_row[c];
     const int p0 = chunk_pair[c], P = chunk_pair[c + 1] - p0;
     unsigned char* reg = region + chunk_off[c];
-    uint32_t* unit = reinterpret_cast<uint32_t*>(reg);
+    uint32_t* run_of = reinterpret_cast<uint32_t*>(reg + ROWS_WARPS);
     int32_t* pr = reinterpret_cast<int32_t*>(reg + region_pr_offset(n, P));
     unsigned long long* kk = key + p0;
     // key (i1, row - r0, e) of each pair (i1 < 64, row - r0 < 2^16, e < 2^30), by insertion
@@ -259,9 +256,8 @@ __global__ void plan_sort(const int32_t* __restrict__ dofmap, const int32_t* __r
       kk[q] = kv;
     }
     // each class: its pairs (the pairs of a row get ranks 0, 1, ..., emitted by (rank,
-    // row, e)) and its work units
-    const int umax = rows_umax(n);
-    int a = 0, n_units = 0;
+    // row, e)) and its run
+    int a = 0, n_runs = 0, share = 0;
     for (int i = 0; i < n; ++i) {
       int b = a;
       while (b < P && int(kk[b] >> 58) == i) ++b;
@@ -275,11 +271,12 @@ __global__ void plan_sort(const int32_t* __restrict__ dofmap, const int32_t* __r
           if (run == rank) pr[out++] = int32_t((kk[j] & E_MASK) * n + i);
         }
       }
-      for (int k0 = a; k0 < b; k0 += umax)
-        unit[1 + n_units++] = uint32_t(i) | (uint32_t(k0) << 7) | (uint32_t(min(k0 + umax, b)) << 19);
+      if (b > a) {
+        for (; share < ROWS_WARPS && P * share / ROWS_WARPS < b; ++share) reg[share] = (unsigned char)n_runs;
+        run_of[n_runs++] = uint32_t(i) | (uint32_t(a) << 7) | (uint32_t(b) << 19);
+      }
       a = b;
     }
-    unit[0] = uint32_t(n_units);
   }
 }
 
@@ -480,20 +477,18 @@ struct Digits {
       d[0] = int(f >> 21);
     }
   }
-  // the 2-digit value v * 2^ulog through the FP64 pipe's int64 -> double conversion (exact:
-  // |v| < 2^53) and an exponent add for 2^ulog; for chunks whose results stay normal
-  // (fp64_ok), so the other lanes' integer conversions and this one use different pipes
-  __device__ __forceinline__ bool fp64_ok() const { return ulog >= -1022 && ulog <= 980; }
-  __device__ __forceinline__ double value_fp64(const int (&s)[NDIG]) const {
-    static_assert(NDIG <= 2, "FP64-pipe conversion of the 31- or 42-bit sums");
-    if constexpr (NDIG == 1) {
-      const long long bits = __double_as_longlong(static_cast<double>(s[0])) + (static_cast<long long>(ulog) << 52);
-      return __longlong_as_double(s[0] == 0 ? 0ll : bits);
-    } else {
-      const long long v = static_cast<long long>(s[0]) * (1ll << 21) + s[1];
-      const long long bits = __double_as_longlong(static_cast<double>(v)) + (static_cast<long long>(ulog) << 52);
-      return __longlong_as_double(v == 0 ? 0ll : bits);
-    }
+  // whether every nonzero one-digit result stays normal
+  __device__ __forceinline__ bool stays_normal() const { return ulog >= -1022 && ulog <= 980; }
+  // a one-digit sum s * 2^ulog whose result stays normal, in 32-bit integer instructions: the magnitude is normalised to a leading one at bit 31, which
+  // completes the exponent field; exact, zero is a select
+  __device__ __forceinline__ double value_int(int s) const {
+    const unsigned m = unsigned(abs(s));
+    unsigned sh;  // leading zeros; 2^32 - 1 for zero, whose shift gives zero
+    asm("bfind.shiftamt.u32 %0, %1;" : "=r"(sh) : "r"(m));
+    unsigned n;
+    asm("shl.b32 %0, %1, %2;" : "=r"(n) : "r"(m), "r"(sh));
+    const unsigned hi = (n >> 11) + (unsigned(1053 + ulog) << 20) - (sh << 20);
+    return __hiloint2double(s == 0 ? 0 : int(hi | (unsigned(s) & 0x80000000u)), int(n << 21));
   }
   // the entry's value from its digit sums, rounded once to FP64
   __device__ __forceinline__ double value(const int (&s)[NDIG]) const {
@@ -510,6 +505,12 @@ struct Digits {
 
 // ---------------------------------------------------------------- geometry
 
+// The three launches of a call are a chain (geometry, bounds, rows); each kernel lets the next
+// one be placed while it runs and waits for the one before where it first needs its results,
+// which takes the launch gaps out of small calls.
+__device__ __forceinline__ void grid_let_next() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+__device__ __forceinline__ void grid_wait_before() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+
 // Form codes of the row kernels: FFC_MASS, FFC_POISSON, or the (mass, Poisson) pair.
 constexpr int ROWS_PAIR = FFC_PAIR_MASS_POISSON;
 
@@ -518,12 +519,13 @@ struct RowsGeo {
   static constexpr int NF = FORM == ROWS_PAIR ? 2 : 1;        // matrices
   static constexpr int NP = D * (D + 1) / 2;                  // symmetric Poisson G_K entries
   static constexpr int NAK = FORM == FFC_POISSON ? NP : 1;    // G entries of a single form
-  // stored per cell: mass [|det|, |det|]; Poisson [G (NP), sum|G|, pad to 8];
-  // pair [|det|, G (NP), pad, sum|G| in slot 7]
+  // stored per cell: mass [|det|, |det|]; Poisson [G (NP), pad, sum|G| in slot 7]; pair [G (NP),
+  // pad, |det| in slot 6, sum|G| in slot 7]
   static constexpr int GS = FORM == FFC_MASS ? 2 : 8;
+  static constexpr int DET = FORM == ROWS_PAIR ? 6 : 0;
   // G_K slots of the contribution bounds' sums: |G| of a single form, and for the pair the
-  // mass's |det J| (slot 0) and the Poisson sum|G| (slot 7)
-  static constexpr int SUM_A = FORM == ROWS_PAIR ? 0 : (FORM == FFC_POISSON ? NP : 1);
+  // mass's |det J| and the Poisson sum|G|, side by side for one load
+  static constexpr int SUM_A = FORM == ROWS_PAIR ? DET : (FORM == FFC_POISSON ? 7 : 1);
   static constexpr int SUM_B = 7;
 };
 
@@ -536,34 +538,35 @@ __global__ void __launch_bounds__(256) rows_geometry(const int32_t* __restrict__
                                                      const double* __restrict__ vertices, long long n_vert,
                                                      long long n_elem, T* __restrict__ G, unsigned* status) {
   using C = RowsGeo<D, FORM>;
+  grid_let_next();
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n_elem;
        e += (long long)gridDim.x * blockDim.x) {
     T g[C::GS];
 #pragma unroll
     for (int a = 0; a < C::GS; ++a) g[a] = T(0);
     bool degenerate = false, bad_index = false;
-    if constexpr (FORM == FFC_MASS || FORM == ROWS_PAIR) {
+    if constexpr (FORM == FFC_MASS || (FORM == ROWS_PAIR && sizeof(T) == 8)) {
       double det;
       cell_det<D>(cells, vertices, n_vert, e, det, degenerate, bad_index);
-      g[0] = T(det);
+      g[C::DET] = T(det);
       if constexpr (FORM == FFC_MASS) g[1] = fabs(g[0]);
     }
     if constexpr (FORM == FFC_POISSON || FORM == ROWS_PAIR) {
-      constexpr int o = FORM == ROWS_PAIR ? 1 : 0;
       bool dg, bi;
       if constexpr (sizeof(T) == 4) {
         float K[D][D], det;
         cell_geometry_f32<D>(cells, vertices, n_vert, e, K, det, dg, bi);
-        geometry_tensor_f32<D, FFC_POISSON, 1, true>(K, det, nullptr, 0.0, 0.0, reinterpret_cast<float*>(g) + o);
+        if constexpr (FORM == ROWS_PAIR) g[C::DET] = det;  // the mass's |det J|, as cell_det rounds it
+        geometry_tensor_f32<D, FFC_POISSON, 1, true>(K, det, nullptr, 0.0, 0.0, reinterpret_cast<float*>(g));
       } else {
         double K[D][D], det;
         cell_geometry<D>(cells, vertices, n_vert, e, K, det, dg, bi);
-        geometry_tensor_k<D, FFC_POISSON, 1>(K, det, nullptr, 0.0, 0.0, [&](int a, double v) { g[o + a] = T(v); });
+        geometry_tensor_k<D, FFC_POISSON, 1>(K, det, nullptr, 0.0, 0.0, [&](int a, double v) { g[a] = T(v); });
       }
       T s = T(0);
 #pragma unroll
-      for (int a = 0; a < C::NP; ++a) s += fabs(g[o + a]);
-      g[FORM == ROWS_PAIR ? C::SUM_B : C::NP] = s;
+      for (int a = 0; a < C::NP; ++a) s += fabs(g[a]);
+      g[7] = s;
       degenerate |= dg;
       bad_index |= bi;
     }
@@ -593,10 +596,13 @@ struct RowsParams {
   const int32_t* chunk_pair;
   const int64_t* chunk_val;
   const int32_t* chunk_inc;
+  int2* chunk_eb;  // bound exponents of the chunk's forms (ROWS_NO_BOUND: not finite)
   const unsigned char* region;
   const void* G;
   const void* a0a;  // mass or single-form reference tensor [N][NAK][N] in T
   const void* a0b;  // pair: the Poisson reference tensor [N][NP][N]
+  const void* ma;   // largest |A0| entry of each row i1 (the bounds' factor), of either tensor
+  const void* mb;
   double* out_a;
   double* out_b;
   long long n_chunks;
@@ -606,47 +612,42 @@ struct RowsParams {
   unsigned* status;
 };
 
-__host__ __device__ constexpr int gcd_c(int a, int b) { return b == 0 ? a : gcd_c(b, a % b); }
-
-#ifndef ROWS_WB
-#define ROWS_WB 256
-#endif
-#ifndef ROWS_TB
-#define ROWS_TB 256
-#endif
-
 template <int D, int FORM, int Q>
 struct RowsCfg {
   static constexpr int N = nscalar(D, Q);
-  static constexpr bool MAIN = N >= 32;              // lane l takes column l of every pair
-  static constexpr int W = MAIN ? N - 32 : N;        // columns spread over the lanes in order
-  static constexpr int I0 = MAIN ? 32 : 0;           // first of those columns
-  static constexpr int PER = W > 0 ? W / gcd_c(32, W) : 1;  // steps after which a lane's column repeats
+  static constexpr bool MAIN = N >= 32;          // lane l takes column l of every pair
+  static constexpr int W = MAIN ? N - 32 : 0;    // columns beyond the first 32, spread over the lanes
+  static constexpr int PP = MAIN ? 1 : 32 / N;   // pairs a warp takes side by side, N lanes each
+  static constexpr int TP = W > 0 ? 32 / W : 1;  // pairs of a column tail's step
   static constexpr int NP = D * (D + 1) / 2;
   static constexpr int NA = FORM == ROWS_PAIR ? 1 + NP : (FORM == FFC_POISSON ? NP : 1);  // A0 values per entry
   static constexpr int NG = FORM == FFC_MASS ? 1 : 8;  // G_K values read per pair (vector loads)
-  static constexpr int TB = ROWS_TB;    // items of one task of the columns beyond the first 32
-  // Order of an iteration's tasks after the staging ones: for n >= 32 (lane per column)
-  // the work units first and the write-out blocks, shorter (128 indices), last, so that
-  // the iteration ends on short tasks (P4 tets: mass + Poisson 4.28 -> 4.04 ms at 48^3);
-  // otherwise units and write-out blocks alternate while both last (P3: 1.64 ms, 1.69
-  // units first)
-  static constexpr bool UNITS_FIRST = MAIN;
-  static constexpr int WB = MAIN ? 128 : ROWS_WB;  // digit indices of one write-out task
 };
 
-// A0 entry (i1, i2) of the kernel's form(s), in the order the contraction uses, from the
-// [i1][alpha][i2] copies (lanes of consecutive i2 read consecutive words)
+// A0 entry (i1, i2) of the kernel's form(s), in the order the contraction uses: mass and FP64
+// from the [i1][alpha][i2] copies (lanes of consecutive i2 read consecutive words), FP32
+// Poisson from the padded rows [i1][i2][alpha], in two vector loads instead of six
 template <int FORM, int N, int NA, int NP, typename T>
 __device__ __forceinline__ void load_a0(const T* __restrict__ A0a, const T* __restrict__ A0b, int i1, int i2,
                                         T (&a)[NA]) {
-  if constexpr (FORM == ROWS_PAIR) {
+  if constexpr (FORM == FFC_MASS) {
     a[0] = __ldg(A0a + i1 * N + i2);
-#pragma unroll
-    for (int j = 0; j < NP; ++j) a[1 + j] = __ldg(A0b + (i1 * NP + j) * N + i2);
   } else {
+    constexpr int o = FORM == ROWS_PAIR ? 1 : 0;
+    if constexpr (o) a[0] = __ldg(A0a + i1 * N + i2);
+    const T* A0p = o ? A0b : A0a;
+    if constexpr (sizeof(T) == 4) {  // [i1][i2][NP padded to 16 bytes]
+      const float4* r = reinterpret_cast<const float4*>(A0p) + (i1 * N + i2) * ((NP + 3) / 4);
+      const float4 x = __ldg(r);
+      a[o] = x.x, a[o + 1] = x.y, a[o + 2] = x.z;
+      if constexpr (NP > 3) {
+        const float2 y = __ldg(reinterpret_cast<const float2*>(r + 1));
+        a[o + 3] = x.w, a[o + 4] = y.x, a[o + 5] = y.y;
+      }
+    } else {
 #pragma unroll
-    for (int j = 0; j < NA; ++j) a[j] = __ldg(A0a + (i1 * NA + j) * N + i2);
+      for (int j = 0; j < NP; ++j) a[o + j] = __ldg(A0p + (i1 * NP + j) * N + i2);
+    }
   }
 }
 
@@ -673,10 +674,10 @@ __device__ __forceinline__ void load_gk(const T* gs, T (&g)[NG]) {
 template <int FORM, int NA, int NG, int NF, typename T>
 __device__ __forceinline__ void contract(const T (&g)[NG], const T (&a)[NA], T (&v)[NF]) {
   if constexpr (FORM == ROWS_PAIR) {
-    v[0] = fma(g[0], a[0], T(0));
+    v[0] = fma(g[6], a[0], T(0));  // |det J| sits in slot 6
     T s = T(0);
 #pragma unroll
-    for (int j = 1; j < NA; ++j) s = fma(g[j], a[j], s);
+    for (int j = 1; j < NA; ++j) s = fma(g[j - 1], a[j], s);
     v[1] = s;
   } else {
     T s = T(0);
@@ -712,93 +713,165 @@ __device__ __forceinline__ void add_digits(int* const (&base)[NF], const Digits<
 // the plan was built, so q < V); the mask only keeps a shared-memory index in range.
 __device__ __forceinline__ int rows_pos(int q) { return q & (ROWS_VMAX - 1); }
 
-#ifndef ROWS_UNROLL
-#define ROWS_UNROLL 2
-#endif
-constexpr int kRowsUnroll = ROWS_UNROLL;  // pairs of a work unit in flight per loop step
-
-
-
-// One work unit (class i1, pairs [k0, k1)) of a chunk, by one warp: for n >= 32 lane l takes
-// column l of every pair (the A0 column in registers), for n < 32 the unit's (pair, column)
-// items in order.
+// Pairs [k0, k1) of class i1 of a chunk, by one warp: for n >= 32 lane l takes column l of
+// every pair, for n < 32 the warp takes 32 / n pairs side by side, n lanes each; the lane's
+// A0 column stays in registers. (With the (pair, column) items packed over all 32 lanes
+// each step divided by n and a lane held the A0 columns of lcm(32, n) / 32 steps: P4
+// triangles 628 against 220 us on 180,000 cells.)
 template <class K, int FORM, int NF, int GS, bool MAGIC, int NDIG, typename T>
-__device__ __forceinline__ void unit_task(unsigned ud, const T* gs, const uint16_t* pos, int* const (&base)[NF],
-                                          const Digits<NDIG> (&dig)[NF], const T* A0a, const T* A0b) {
-  constexpr int N = K::N, NA = K::NA, NG = K::NG;
-  const int lane = threadIdx.x & 31;
-  const int i1 = int(ud & 127u), k0 = int((ud >> 7) & 4095u), k1 = int(ud >> 19);
-  if constexpr (K::MAIN) {
-    T am[NA];
-    load_a0<FORM, N, NA, K::NP, T>(A0a, A0b, i1, lane, am);
-    const uint16_t* pl = pos + lane;
-#pragma unroll kRowsUnroll
-    for (int k = k0; k < k1; ++k) {
-      T g[NG];
-      load_gk<NG, T>(gs + k * GS, g);
-      const int q = rows_pos(pl[k * N]);
-      T v[NF];
-      contract<FORM, NA, NG, NF, T>(g, am, v);
-      add_digits<MAGIC, NF, NDIG, T>(base, dig, v, q);
-    }
-  } else {
-    T af[K::PER][NA];
-#pragma unroll
-    for (int s = 0; s < K::PER; ++s) load_a0<FORM, N, NA, K::NP, T>(A0a, A0b, i1, (lane + 32 * s) % K::W, af[s]);
-    const int total = (k1 - k0) * K::W;
-    for (int f0 = 0; f0 < total; f0 += 32 * K::PER) {
-#pragma unroll
-      for (int s = 0; s < K::PER; ++s) {
-        const int f = f0 + 32 * s + lane;
-        if (f < total) {
-          const int kk = k0 + f / K::W;
-          const int i2 = K::I0 + f % K::W;
-          T g[NG];
-          load_gk<NG, T>(gs + kk * GS, g);
-          const int q = rows_pos(pos[kk * N + i2]);
-          T v[NF];
-          contract<FORM, NA, NG, NF, T>(g, af[s], v);
-          add_digits<MAGIC, NF, NDIG, T>(base, dig, v, q);
-        }
-      }
-    }
-  }
-}
-
-// Items [b * TB, (b + 1) * TB) of the columns beyond the first 32 (n > 32), packed over
-// the lanes: item f is pair f / W, column 32 + f % W.
-template <class K, int FORM, int NF, int GS, bool MAGIC, int NDIG, typename T>
-__device__ __forceinline__ void tail_task(int b, int P, const int32_t* pr, const T* gs, const uint16_t* pos,
+__device__ __forceinline__ void run_pairs(int i1, int k0, int k1, const T* gs, const uint16_t* pos,
                                           int* const (&base)[NF], const Digits<NDIG> (&dig)[NF], const T* A0a,
                                           const T* A0b) {
   constexpr int N = K::N, NA = K::NA, NG = K::NG;
-  if constexpr (K::MAIN && K::W > 0) {
-    const int total = P * K::W, end = min(total, (b + 1) * K::TB);
-    for (int f = b * K::TB + (threadIdx.x & 31); f < end; f += 32) {
-      const int k = f / K::W, i2 = 32 + f % K::W;
-      const int i1 = pr[k] % N;
+  const int lane = threadIdx.x & 31;
+  const int sub = K::MAIN ? 0 : lane / N, i2 = K::MAIN ? lane : lane - sub * N;
+  if (sub >= K::PP) return;
+  T am[NA];
+  load_a0<FORM, N, NA, K::NP, T>(A0a, A0b, i1, i2, am);
+  const uint16_t* pl = pos + i2;
+#pragma unroll 3
+  for (int k = k0 + sub; k < k1; k += K::PP) {
+    T g[NG];
+    load_gk<NG, T>(gs + k * GS, g);
+    const int q = rows_pos(pl[k * N]);
+    T v[NF];
+    contract<FORM, NA, NG, NF, T>(g, am, v);
+    add_digits<MAGIC, NF, NDIG, T>(base, dig, v, q);
+  }
+}
+
+// One warp's share [k0, k1) of a chunk's pairs: the class runs it meets, from run r on.
+template <class K, int FORM, int NF, int GS, bool MAGIC, int NDIG, typename T>
+__device__ __forceinline__ void share_task(int r, int k0, int k1, const unsigned* run, const int32_t* pr, const T* gs,
+                                           const uint16_t* pos,
+                                            int* const (&base)[NF], const Digits<NDIG> (&dig)[NF], const T* A0a,
+                                           const T* A0b) {
+  if constexpr (sizeof(T) == 8 && !K::MAIN && K::PP * K::N < 28) {
+    // the FP64 pipe takes as long for 20 lanes as for 32 (P3 tetrahedra): the share's
+    // (pair, column) items packed over all lanes, A0 from the L1 cache
+    constexpr int N = K::N, NA = K::NA, NG = K::NG;
+#pragma unroll 1
+    for (int f = threadIdx.x & 31; f < (k1 - k0) * N; f += 32) {
+      const int k = k0 + f / N, i2 = f % N;
       T a[NA], g[NG];
-      load_a0<FORM, N, NA, K::NP, T>(A0a, A0b, i1, i2, a);
+      load_a0<FORM, N, NA, K::NP, T>(A0a, A0b, pr[k] % N, i2, a);
       load_gk<NG, T>(gs + k * GS, g);
       const int q = rows_pos(pos[k * N + i2]);
       T v[NF];
       contract<FORM, NA, NG, NF, T>(g, a, v);
       add_digits<MAGIC, NF, NDIG, T>(base, dig, v, q);
     }
+    return;
+  }
+  for (int k = k0; k < k1; ++r) {
+    const unsigned ud = run[r];
+    const int end = min(k1, int(ud >> 19));
+    run_pairs<K, FORM, NF, GS, MAGIC, NDIG, T>(int(ud & 127u), k, end, gs, pos, base, dig, A0a, A0b);
+    k = end;
   }
 }
 
-// Per-chunk state prepared one iteration ahead (three slots, by chunk index mod 3), read by
-// every warp of the iteration that uses it.
-template <int NDIG>
-struct RowsSlot {
-  Digits<NDIG> dig[2];  // fixed-point digits of each form (from its bound's exponent)
-  int finite[2];        // the form's bound is finite
-  int shift[2];         // chunk position q of form f sits at digit index q + shift[f]: the
-                        // output address of index 0 is then 16-byte aligned
-  int n_units, n_items;  // work units, and units + column-tail blocks
-  int P, V;              // pairs and CSR values of the chunk
+// The columns beyond the first 32 (n > 32) of pairs [step TP, (step + 1) TP) of a chunk,
+// packed over the lanes, W to a pair.
+template <class K, int FORM, int NF, int GS, bool MAGIC, int NDIG, typename T>
+__device__ __forceinline__ void tail_step(int step, int P, const int32_t* pr, const T* gs, const uint16_t* pos,
+                                          int* const (&base)[NF], const Digits<NDIG> (&dig)[NF], const T* A0a,
+                                          const T* A0b) {
+  constexpr int N = K::N, NA = K::NA, NG = K::NG, TP = K::TP;
+  const int lane = threadIdx.x & 31, sub = lane / K::W, i2 = 32 + lane - sub * K::W;
+  const int k = step * TP + sub;
+  if (sub >= TP || k >= P) return;
+  T a[NA], g[NG];
+  load_a0<FORM, N, NA, K::NP, T>(A0a, A0b, pr[k] % N, i2, a);
+  load_gk<NG, T>(gs + k * GS, g);
+  const int q = rows_pos(pos[k * N + i2]);
+  T v[NF];
+  contract<FORM, NA, NG, NF, T>(g, a, v);
+  add_digits<MAGIC, NF, NDIG, T>(base, dig, v, q);
+}
+
+// The bound exponents of every chunk, before the rows: a warp per chunk takes the largest
+// contribution bound of its pairs (max|A0[i1][.][.]| sum|G_K|) times the most pairs of a row,
+// and 2^(eb-1) is that or the next power of two. In rows_assemble one warp did this for a
+// later chunk in every iteration and its chain of loads and shuffles was the iteration's
+// shortest possible time (235 of 443 us for P4 pair rows of 82,944 tets with no other work);
+// here all chunks run side by side.
+constexpr int ROWS_NO_BOUND = INT_MAX;  // the bound is not finite
+
+template <int D, int FORM, int Q, typename T>
+__global__ void __launch_bounds__(256) rows_bounds(RowsParams p) {
+  using C = RowsGeo<D, FORM>;
+  using K = RowsCfg<D, FORM, Q>;
+  constexpr int N = K::N, NF = C::NF;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const T big = sizeof(T) == 4 ? T(FLT_MAX) : T(DBL_MAX);
+  const T* M[2] = {static_cast<const T*>(p.ma), static_cast<const T*>(p.mb)};
+  grid_let_next();
+  const T* G = static_cast<const T*>(p.G);
+  bool waited = false;
+  for (long long c = blockIdx.x * 8ll + w; c < p.n_chunks; c += gridDim.x * 8ll) {
+    // the plan's part first, all of the lane's pairs at once: only the geometry has to wait
+    const int P = p.chunk_pair[c + 1] - p.chunk_pair[c];
+    const int32_t* pr = reinterpret_cast<const int32_t*>(p.region + p.chunk_off[c] + region_pr_offset(N, P));
+    constexpr int PL = ROWS_PMAX / 32;
+    int t[PL];
+#pragma unroll
+    for (int j = 0; j < PL; ++j) t[j] = lane + 32 * j < P ? __ldg(pr + lane + 32 * j) : -1;
+    if (!waited) grid_wait_before();
+    waited = true;
+    T pb[NF];
+#pragma unroll
+    for (int f = 0; f < NF; ++f) pb[f] = T(0);
+#pragma unroll
+    for (int j = 0; j < PL; ++j) {
+      if (t[j] < 0) continue;
+      const int e = t[j] / N, i1 = t[j] - e * N;
+      const T* g = G + (long long)e * C::GS + C::SUM_A;
+      T s[NF];
+      if constexpr (NF == 1) {
+        s[0] = *g;
+      } else {
+        using V = typename std::conditional<sizeof(T) == 4, float2, double2>::type;
+        const V v = *reinterpret_cast<const V*>(g);
+        s[0] = v.x, s[1] = v.y;
+      }
+#pragma unroll
+      for (int f = 0; f < NF; ++f) {
+        const T x = __ldg(M[f] + i1) * fabs(s[f]);
+        pb[f] = fmax(pb[f], x == x ? x : big * T(2));  // NaN -> inf
+      }
+    }
+    int eb[2] = {0, 0};
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+      const T bnd = warp_max(pb[f]) * T(p.chunk_inc[c]);
+      eb[f] = bnd <= big ? bound_exponent(bnd) : ROWS_NO_BOUND;
+    }
+    if (lane == 0) p.chunk_eb[c] = make_int2(eb[0], eb[1]);
+  }
+}
+
+// State of one chunk, prepared some iterations ahead by one warp and read with 16-byte loads.
+struct __align__(16) RowsForm {  // of one form
+  double* out;                   // output of digit index 0: the chunk's first value - shift
+  int eb;                        // bound exponent (ROWS_NO_BOUND: not finite)
+  int shift;                     // chunk position q sits at digit index q + shift: index 0 is
+                                 // then at a 16-byte aligned output address
 };
+struct __align__(16) RowsChunk {
+  RowsForm form[2];
+  long long region;  // byte offset of its region
+  int P, V;          // pairs, CSR values
+  int bytes, pad[3]; // of the region
+};
+__device__ __forceinline__ RowsForm rows_form(const RowsChunk& c, int f) {
+  const int4 v = *reinterpret_cast<const int4*>(&c.form[f]);
+  RowsForm r;
+  r.out = reinterpret_cast<double*>(static_cast<unsigned long long>(unsigned(v.y)) << 32 | unsigned(v.x));
+  r.eb = v.z;
+  r.shift = v.w;
+  return r;
+}
 
 // mbarrier helpers of the staging copies: cp.async issued by one warp, tracked by an
 // mbarrier of arrival count 32 (each lane arrives when its own copies have landed)
@@ -826,24 +899,19 @@ __device__ __forceinline__ bool rows_bar_wait(unsigned long long* bar, unsigned 
   return false;
 }
 
-// Values (of each 4 consecutive ones a lane converts) that take the FP64 pipe's integer
-// conversion where it is exact: bit c set for value c.
-#ifndef ROWS_FP64_MASK
-#define ROWS_FP64_MASK 0xA
-#endif
-
-// The chunks of this CTA are c_i = blockIdx.x + i * gridDim.x. Iteration i is one queue of
-// independent warp tasks, handed out by a shared counter: three staging tasks (chunk i + 3's
-// plan region, chunk i + 2's geometry and digits, chunk i + 5's extents), then the work
-// units of chunk i (into accumulator buffer i % 2) interleaved with the write-out blocks of
-// chunk i - 1 (from the other buffer, which they clear). The region copy is cp.async
-// tracked by an mbarrier that only its consumer (the geometry task, an iteration later)
-// waits for; the geometry task gathers the pairs' G_K, waits for its own copies, and
-// derives the chunk's fixed-point digits from the largest contribution bound. The work
-// units come with the plan. One CTA-wide barrier closes each iteration. Staging depths:
-// regions 4 buffers (i .. i + 3), geometry 3 (i .. i + 2), per-chunk state 4 slots
-// (i - 1 .. i + 2), extents a ring of 8. A wait that gives up sets FFC_FLAG_TIMEOUT and
-// ends the CTA's work after the iteration.
+// The chunks of this CTA are c_i = blockIdx.x + i * gridDim.x. In iteration i every warp sums
+// its equal share of chunk i's pairs (into accumulator buffer i % 2) and writes its blocks of
+// chunk i - 1's values (from the other buffer, which it clears); odd warps write first, so
+// the warps of a scheduler mix the shared-memory atomics of one with the conversions of the
+// other. Staging runs beside it: warps 0-7 copy chunk i + 3's plan region, warps 8-15 gather
+// the G_K of chunk i + 2's pairs (its region was asked for an iteration earlier) and warp 16
+// prepares the state of chunk i + 5. The copies are cp.async, tracked by mbarriers that
+// their readers wait for an iteration or two later, so no warp waits for memory. One
+// CTA-wide barrier closes each iteration. (A queue of warp tasks instead, units of up to 16
+// pairs and 128-value blocks handed out by a shared counter, took 1.65 us an iteration on
+// fetching and staging alone.) Staging depths: regions 4 buffers (i .. i + 3), geometry 3
+// (i .. i + 2), chunk states a ring of 8 (i - 1 .. i + 5). A wait that gives up sets
+// FFC_FLAG_TIMEOUT and ends the CTA's work after the iteration.
 // One CTA per SM: 32 warps for FP32 (64 registers a thread), 16 for FP64.
 template <int D, int FORM, int Q, typename T>
 __global__ void __launch_bounds__(sizeof(T) == 4 ? 1024 : 512, 1) rows_assemble(RowsParams p) {
@@ -852,81 +920,81 @@ __global__ void __launch_bounds__(sizeof(T) == 4 ? 1024 : 512, 1) rows_assemble(
   constexpr int N = K::N, NF = C::NF, GS = C::GS, TH = sizeof(T) == 4 ? 1024 : 512;
   constexpr int NDIG = rows_ndig<T>();  // digits: 31-bit fixed point for FP32, 63-bit for FP64
   constexpr int ACC = NF * NDIG * ROWS_VSTRIDE;  // ints of one accumulator buffer
-  constexpr int NSPECIAL = 3;
-  using Slot = RowsSlot<NDIG>;
+  constexpr int NW = TH / 32, SW = NW / 4;  // warps; of one staging job
   extern __shared__ __align__(16) unsigned char smem[];
   int* acc = reinterpret_cast<int*>(smem);                                   // [2][NF][NDIG][ROWS_VSTRIDE]
   unsigned char* rbuf = smem + size_t(2) * ACC * 4;                          // [4][rmax] plan regions
   T* gbuf = reinterpret_cast<T*>(rbuf + 4 * size_t(p.rmax));                 // [3][pmax][GS]
-  T* a0max = gbuf + 3 * size_t(p.pmax) * GS;                                 // [NF][N]
-  Slot* slot = reinterpret_cast<Slot*>(a0max + NF * N);                      // [4]
-  int* tq = reinterpret_cast<int*>(slot + 4);                                // [2] task counters, [2] abort
-  long long* meta = reinterpret_cast<long long*>(smem + p.meta_off);          // [8][8]: chunk extents
-  unsigned long long* rbar = reinterpret_cast<unsigned long long*>(meta + 64);  // [4] region copies
+  RowsChunk* ring = reinterpret_cast<RowsChunk*>(smem + p.meta_off);          // [8] chunk states
+  unsigned long long* rbar = reinterpret_cast<unsigned long long*>(ring + 8);  // [4] region copies
+  unsigned long long* gbar = rbar + 4;                                          // [3] geometry copies
   const T* A0a = static_cast<const T*>(p.a0a);
   const T* A0b = static_cast<const T*>(p.a0b);
   const T* Gall = static_cast<const T*>(p.G);
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-  const T big = sizeof(T) == 4 ? T(FLT_MAX) : T(DBL_MAX);
   const int G1 = int(gridDim.x);
   const int n_iter = blockIdx.x < p.n_chunks ? int((p.n_chunks - blockIdx.x + G1 - 1) / G1) : 0;
-  // largest |A0| entry of each reference-tensor row i1 (the contribution bound's factor)
-  for (int i = t; i < NF * N; i += TH) {
-    const int f = i / N, i1 = i - f * N;
-    const int na = (FORM == ROWS_PAIR && f == 1) ? C::NP : C::NAK;
-    const T* A = (FORM == ROWS_PAIR && f == 1) ? A0b : A0a;
-    T m = T(0);
-    for (int k = 0; k < N * na; ++k) m = fmax(m, fabs(A[size_t(i1) * N * na + k]));
-    a0max[i] = m;
-  }
   for (int i = 4 * t; i < 2 * ACC; i += 4 * TH) *reinterpret_cast<int4*>(acc + i) = make_int4(0, 0, 0, 0);
-  if (t < 3) tq[t] = 0;
-  if (t < 4) rows_bar_init(rbar + t, 32);
-  // extents of the chunk of iteration i, ring slot i % 8: pairs [0] .. [1), region bytes
-  // [2] .. [3), CSR values [4] .. [5), most pairs of a row [6]
-  auto meta_at = [&](int i) { return meta + (i & 7) * 8; };
-  auto meta_task = [&](int i) {  // one warp
-    const long long c = blockIdx.x + (long long)i * G1;
-    if (i < n_iter && lane < 7) {
-      long long v;
+  if (t < 7) rows_bar_init(rbar + t, 32 * SW);
+  bool failed = false;  // a wait of this warp gave up
+  auto give_up = [&]() {
+    if (lane == 0) atomicOr(p.status, FFC_FLAG_TIMEOUT);
+    failed = true;
+  };
+  auto chunk_at = [&](int i) -> RowsChunk& { return ring[i & 7]; };
+  // the state of iteration i's chunk into ring slot i % 8, by one warp: lanes 0-6 load its
+  // extents and exponents, lanes 0 and 1 derive each form's part
+  auto chunk_load = [&](int i) {
+    long long v = 0;
+    if (i < n_iter) {
+      const long long c = blockIdx.x + (long long)i * G1;
       if (lane < 2) v = p.chunk_pair[c + lane];
       else if (lane < 4) v = p.chunk_off[c + lane - 2];
       else if (lane < 6) v = p.chunk_val[c + lane - 4];
-      else v = p.chunk_inc[c];
-      meta_at(i)[lane] = v;
+      else if (lane < 7) v = reinterpret_cast<const long long*>(p.chunk_eb)[c];
+    }
+    return v;
+  };
+  auto chunk_store = [&](int i, long long v) {
+    auto from = [&](int l) { return __shfl_sync(0xffffffffu, v, l); };
+    const int P = int(from(1) - from(0));
+    const long long r0 = from(2), r1 = from(3), v0 = from(4), v1 = from(5), ebs = from(6);
+    RowsChunk& ch = chunk_at(i);
+    if (lane < NF) {
+      const int eb = int(lane == 0 ? ebs : ebs >> 32);
+      double* out = (lane == 0 ? p.out_a : p.out_b) + v0;
+      const int sh = int((reinterpret_cast<uintptr_t>(out) >> 3) & 1);
+      ch.form[lane].out = out - sh;
+      ch.form[lane].eb = eb;
+      ch.form[lane].shift = sh;
+    }
+    if (lane == 2) {
+      ch.region = r0;
+      ch.bytes = int(r1 - r0);
+      ch.P = P;
+      ch.V = int(v1 - v0);
     }
   };
   auto region_at = [&](int i) { return rbuf + (i & 3) * p.rmax; };
   auto geom_at = [&](unsigned i3) { return gbuf + i3 * p.pmax * GS; };  // i3 = i % 3
   // the plan region of chunk i (a multiple of 16 bytes, at most rmax) into buffer i % 4
-  auto region_task = [&](int i) {  // one warp
-    const long long* m = meta_at(i);
-    const unsigned char* src = p.region + m[2];
+  auto region_task = [&](int i, int part) {  // part of SW warps
+    const unsigned char* src = p.region + chunk_at(i).region;
     unsigned char* dst = region_at(i);
-    const int nb = int(m[3] - m[2]);
-    for (int o = 16 * lane; o < nb; o += 512) cp_async16(dst + o, src + o);
+    const int nb = chunk_at(i).bytes;
+    for (int o = 16 * (part * 32 + lane); o < nb; o += 512 * SW) cp_async16(dst + o, src + o);
     rows_cp_async_arrive(rbar + (i & 3));
   };
-  // chunk i's geometry (one warp, once its region has landed): the pairs' G_K gathered
-  // into buffer i % 3, then its per-chunk state in slot i % 4: fixed-point digits from the
-  // bound (largest pair bound times the most pairs of a row), output alignment shifts,
-  // counts
-  auto geometry_task = [&](int i) {
-    Slot& sl = slot[i & 3];
+  // the G_K of chunk i's pairs into buffer i % 3 (once the region has landed)
+  auto geometry_task = [&](int i, int part) {  // part of SW warps
     if (!rows_bar_wait(rbar + (i & 3), unsigned(i >> 2) & 1u)) {
-      if (lane == 0) {
-        atomicOr(p.status, FFC_FLAG_TIMEOUT);
-        tq[2] = 1;
-        sl.n_units = sl.n_items = sl.P = sl.V = 0;
-      }
+      give_up();
       return;
     }
-    const long long* m = meta_at(i);
-    const int P = int(m[1] - m[0]);
-    const unsigned char* reg = region_at(i);
-    const int32_t* pr = reinterpret_cast<const int32_t*>(reg + region_pr_offset(N, P));
+    const int P = chunk_at(i).P;
+    const int32_t* pr = reinterpret_cast<const int32_t*>(region_at(i) + region_pr_offset(N, P));
     T* gs = geom_at(unsigned(i) % 3u);
-    for (int k = lane; k < P; k += 32) {
+    for (int k = part * 32 + lane; k < P; k += 32 * SW) {
       const T* src = Gall + (long long)(pr[k] / N) * GS;
       if constexpr (GS * sizeof(T) == 8) {
         cp_async8(gs + k * GS, src);
@@ -937,188 +1005,147 @@ __global__ void __launch_bounds__(sizeof(T) == 4 ? 1024 : 512, 1) rows_assemble(
                      reinterpret_cast<const unsigned char*>(src) + 16 * x);
       }
     }
-    cp_async_commit();
-    cp_async_wait_all();
-    __syncwarp();
-    T pb[NF];
-#pragma unroll
-    for (int f = 0; f < NF; ++f) pb[f] = T(0);
-    for (int k = lane; k < P; k += 32) {
-      const int i1 = pr[k] % N;
-#pragma unroll
-      for (int f = 0; f < NF; ++f) {
-        const T x = a0max[f * N + i1] * fabs(gs[k * GS + (f == 0 ? C::SUM_A : C::SUM_B)]);
-        pb[f] = fmax(pb[f], x == x ? x : big * T(2));  // NaN -> inf
-      }
-    }
-#pragma unroll
-    for (int f = 0; f < NF; ++f) {
-      const T bnd = warp_max(pb[f]) * T(m[6]);
-      if (lane == f) {
-        sl.finite[f] = bnd <= big;
-        Digits<NDIG> dg;
-        dg.init(bnd <= big ? bound_exponent(bnd) : 0);
-        sl.dig[f] = dg;
-        const double* out = (f == 0 ? p.out_a : p.out_b) + m[4];
-        sl.shift[f] = int((reinterpret_cast<uintptr_t>(out) >> 3) & 1);
-      }
-    }
-    if (lane == 31) {
-      const int nu = int(*reinterpret_cast<const uint32_t*>(reg));
-      sl.n_units = nu;
-      sl.n_items = nu + (K::MAIN && K::W > 0 ? (P * K::W + K::TB - 1) / K::TB : 0);
-      sl.P = P;
-      sl.V = int(m[5] - m[4]);
-    }
+    rows_cp_async_arrive(gbar + unsigned(i) % 3u);
   };
-  // digit indices [b * WB, (b + 1) * WB) of chunk i from accumulator buffer i % 2 (cleared),
-  // one warp: each lane converts four consecutive indices per step and stores them as two
-  // 16-byte pairs (index x is output value x - shift, and output index 0 is 16-byte
-  // aligned); where the FP64 pipe's conversion is exact, the values of ROWS_FP64_MASK take
-  // it, so two pipes share the conversions
-  auto write_task = [&](int i, int b) {
-    const Slot& sl = slot[i & 3];
-    const long long v0 = meta_at(i)[4];
-    const int V = sl.V;
+  // this warp's digit indices of chunk i, every NW-th 128, from accumulator buffer i % 2
+  // (cleared): a lane converts two consecutive indices at a time and stores them together
+  // (index x is output value x - shift, and output index 0 is 16-byte aligned), so a store
+  // instruction covers 512 consecutive bytes. Two stores of a lane's four consecutive values,
+  // each covering half of every line, cost the L1 data pipe twice the cycles (P4: 3123
+  // against 2998 us); and half of the conversions on the FP64 pipe, 3034 us.
+  auto write_task = [&](int i) {
+    const RowsChunk& ch = chunk_at(i);
+    const int V = ch.V;
     int* ab = acc + (i & 1) * ACC;
-    const double nan = __longlong_as_double(0x7ff8000000000000ll);
 #pragma unroll
     for (int f = 0; f < NF; ++f) {
-      const Digits<NDIG> dg = sl.dig[f];
-      const bool fin = sl.finite[f] != 0;
-      const int sh = sl.shift[f];
-      double* out = (f == 0 ? p.out_a : p.out_b) + v0 - sh;
+      const RowsForm st = rows_form(ch, f);
+      const int eb = st.eb, sh = st.shift;
+      const bool fin = eb != ROWS_NO_BOUND;
+      Digits<NDIG> dg;
+      dg.init(fin ? eb : 0);
+      const bool fast = NDIG == 1 && fin && dg.stays_normal();
+      double* out = st.out;
       int* a = ab + f * NDIG * ROWS_VSTRIDE;
-      const bool split_pipes = NDIG <= 2 && fin && dg.fp64_ok();
-      const int hi = V + sh, end = min(hi, (b + 1) * K::WB);
-      for (int x = b * K::WB + 4 * lane; x < end; x += 128) {
-        int4 dd[NDIG];
-#pragma unroll
-        for (int d = 0; d < NDIG; ++d) {
-          dd[d] = *reinterpret_cast<const int4*>(a + d * ROWS_VSTRIDE + x);
-          *reinterpret_cast<int4*>(a + d * ROWS_VSTRIDE + x) = make_int4(0, 0, 0, 0);
-        }
-        double r[4];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          int sd[NDIG];
-#pragma unroll
-          for (int d = 0; d < NDIG; ++d) sd[d] = c == 0 ? dd[d].x : c == 1 ? dd[d].y : c == 2 ? dd[d].z : dd[d].w;
-          if constexpr (NDIG <= 2) {
-            if (((ROWS_FP64_MASK >> c) & 1) && split_pipes) {
-              r[c] = dg.value_fp64(sd);
-              continue;
-            }
-          }
-          r[c] = fin ? dg.value(sd) : nan;
-        }
+      const int hi = V + sh;
+      for (int x0 = 128 * w + 2 * lane; x0 < hi; x0 += 128 * NW) {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-          const int y = x + 2 * h;
-          if (y >= sh && y + 1 < hi) {
-            __stcs(reinterpret_cast<double2*>(out + y), make_double2(r[2 * h], r[2 * h + 1]));
+          const int x = x0 + 64 * h;
+          if (x >= hi) break;
+          int sd[2][NDIG];
+#pragma unroll
+          for (int d = 0; d < NDIG; ++d) {
+            int2* src = reinterpret_cast<int2*>(a + d * ROWS_VSTRIDE + x);
+            const int2 v = *src;
+            *src = make_int2(0, 0);
+            sd[0][d] = v.x;
+            sd[1][d] = v.y;
+          }
+          double r[2];
+          if (fast) {
+            r[0] = dg.value_int(sd[0][0]);
+            r[1] = dg.value_int(sd[1][0]);
           } else {
-            if (y >= sh && y < hi) __stcs(out + y, r[2 * h]);
-            if (y + 1 >= sh && y + 1 < hi) __stcs(out + y + 1, r[2 * h + 1]);
+#pragma unroll
+            for (int c = 0; c < 2; ++c) r[c] = fin ? dg.value(sd[c]) : __longlong_as_double(0x7ff8000000000000ll);
+          }
+          double* o = out + x;
+          if (x >= sh && x + 1 < hi) {
+            __stcs(reinterpret_cast<double2*>(o), make_double2(r[0], r[1]));
+          } else {
+            if (x >= sh) __stcs(o, r[0]);
+            if (x + 1 >= sh && x + 1 < hi) __stcs(o + 1, r[1]);
           }
         }
       }
     }
   };
-  // ---- prologue: extents of iterations 0..4; regions of chunks 0..2; geometry of chunks
-  // 0..1 (each waits for what it reads)
-  if (w < 5) meta_task(w);
+  grid_wait_before();
+  // ---- prologue: states of chunks 0..4, regions of chunks 0..2, geometry of chunks 0..1
+  if (w < 5) {
+    const long long v = chunk_load(w);
+    if (w < n_iter) chunk_store(w, v);
+  }
   __syncthreads();
-  if (w < 3 && w < n_iter) region_task(w);
-  if (w == 3 && n_iter > 0) geometry_task(0);
-  if (w == 4 && n_iter > 1) geometry_task(1);
+  if (w < 3 * SW && w / SW < n_iter) region_task(w / SW, w % SW);
   __syncthreads();
-  unsigned i3 = 0;  // i % 3
-  for (int i = 0; i <= n_iter && tq[2] == 0; ++i, i3 = i3 == 2 ? 0 : i3 + 1) {
-    if (t == 0) tq[(i + 1) & 1] = 0;  // the next iteration's queue (last used two iterations ago)
-    // this iteration's work: units (and column tails) of chunk i, write-out blocks of chunk i - 1
-    const Slot& cur = slot[i & 3];
-    int nI = 0, nU = 0, nW = 0, P = 0;
+  if (w < 2 * SW && w / SW < n_iter) geometry_task(w / SW, w % SW);
+  if (__syncthreads_or(failed)) {
+    cp_async_commit();
+    cp_async_wait_all();
+    return;
+  }
+  unsigned i3 = 0, gpar = 0;  // i % 3, (i / 3) % 2
+  for (int i = 0; i <= n_iter; ++i) {
+    long long next = 0;
+    if (w < SW) {
+      if (i + 3 < n_iter) region_task(i + 3, w);
+    } else if (w < 2 * SW) {
+      if (i + 2 < n_iter) geometry_task(i + 2, w - SW);
+    } else if (w == 2 * SW) {
+      next = chunk_load(i + 5);
+    }
+    if (i >= 1 && (w & 1)) write_task(i - 1);
     if (i < n_iter) {
-      P = cur.P;
-      nU = cur.n_units;
-      nI = cur.n_items;
-    }
-    if (i >= 1) nW = (slot[(i - 1) & 3].V + 1 + K::WB - 1) / K::WB;  // indices up to V + shift
-    const int nMix = 2 * min(nI, nW), n_tasks = NSPECIAL + nI + nW;
-    const unsigned char* reg = region_at(i);
-    const unsigned* un = reinterpret_cast<const unsigned*>(reg) + 1;
-    const int32_t* pr = reinterpret_cast<const int32_t*>(reg + region_pr_offset(N, P));
-    const uint16_t* pos = reinterpret_cast<const uint16_t*>(reg + region_pr_offset(N, P) + 4 * P);
-    const T* gs = geom_at(i3);
-    int* ab = acc + (i & 1) * ACC;
-    Digits<NDIG> dig[NF];
-    int* base[NF];
-    bool magic = sizeof(T) == 4;
+      if (rows_bar_wait(gbar + i3, gpar)) {  // chunk i's geometry; its region landed before that
+        const RowsChunk& ch = chunk_at(i);
+        const int P = ch.P;
+        const unsigned char* reg = region_at(i);
+        const unsigned* run = reinterpret_cast<const unsigned*>(reg + ROWS_WARPS);
+        const int32_t* pr = reinterpret_cast<const int32_t*>(reg + region_pr_offset(N, P));
+        const uint16_t* pos = reinterpret_cast<const uint16_t*>(reg + region_pr_offset(N, P) + 4 * P);
+        const T* gs = geom_at(i3);
+        Digits<NDIG> dig[NF];
+        int* base[NF];
+        bool magic = sizeof(T) == 4;
 #pragma unroll
-    for (int f = 0; f < NF; ++f) {
-      base[f] = ab + f * NDIG * ROWS_VSTRIDE;
-      if (i < n_iter) {
-        dig[f] = cur.dig[f];
-        magic = magic && dig[f].magic;
-        base[f] += cur.shift[f];
-      }
-    }
-    for (;;) {
-      int k = 0;
-      if (lane == 0) k = atomicAdd(tq + (i & 1), 1);
-      k = __shfl_sync(0xffffffffu, k, 0);
-      if (k >= n_tasks) break;
-      if (k < NSPECIAL) {
-        if (k == 0 && i + 3 < n_iter) region_task(i + 3);
-        if (k == 1 && i + 2 < n_iter) geometry_task(i + 2);
-        if (k == 2) meta_task(i + 5);
-        continue;
-      }
-      k -= NSPECIAL;
-      bool item;
-      int j;
-      if constexpr (K::UNITS_FIRST) {
-        item = k < nI;
-        j = item ? k : k - nI;
-      } else if (k < nMix) {  // items and write-out blocks alternate while both last
-        item = (k & 1) == 0;
-        j = k >> 1;
-      } else {
-        item = nI > nW;
-        j = k - nMix / 2;
-      }
-      if (item) {
-        if (j < nU) {
-          if (magic) unit_task<K, FORM, NF, GS, true, NDIG, T>(un[j], gs, pos, base, dig, A0a, A0b);
-          else unit_task<K, FORM, NF, GS, false, NDIG, T>(un[j], gs, pos, base, dig, A0a, A0b);
-        } else {
-          if (magic) tail_task<K, FORM, NF, GS, true, NDIG, T>(j - nU, P, pr, gs, pos, base, dig, A0a, A0b);
-          else tail_task<K, FORM, NF, GS, false, NDIG, T>(j - nU, P, pr, gs, pos, base, dig, A0a, A0b);
+        for (int f = 0; f < NF; ++f) {
+          const RowsForm st = rows_form(ch, f);
+          dig[f].init(st.eb != ROWS_NO_BOUND ? st.eb : 0);
+          magic = magic && dig[f].magic;
+          base[f] = acc + (i & 1) * ACC + f * NDIG * ROWS_VSTRIDE + st.shift;
         }
+        const int r = reg[w * (ROWS_WARPS / NW)], k0 = P * w / NW, k1 = P * (w + 1) / NW;
+        auto sum = [&](auto m) {
+          constexpr bool M = decltype(m)::value;
+          share_task<K, FORM, NF, GS, M, NDIG, T>(r, k0, k1, run, pr, gs, pos, base, dig, A0a, A0b);
+          // column tails go to the last warps, the first ones stage
+          if constexpr (K::W > 0)
+            for (int st = NW - 1 - w; st * K::TP < P; st += NW)
+              tail_step<K, FORM, NF, GS, M, NDIG, T>(st, P, pr, gs, pos, base, dig, A0a, A0b);
+        };
+        if (magic) sum(std::true_type());
+        else sum(std::false_type());
       } else {
-        write_task(i - 1, j);
+        give_up();
       }
     }
-    __syncthreads();
+    if (i >= 1 && !(w & 1)) write_task(i - 1);
+    if (w == 2 * SW && i + 5 < n_iter) chunk_store(i + 5, next);
+    if (i3 == 2) {
+      i3 = 0;
+      gpar ^= 1;
+    } else {
+      ++i3;
+    }
+    if (__syncthreads_or(failed)) break;
   }
   cp_async_commit();
   cp_async_wait_all();  // copies of chunks this CTA no longer needed (a wait that gave up)
 }
 
 template <int D, int FORM, int Q, typename T>
-int launch_rows_t(const ffc_row_plan* plan, const void* a0a, const void* a0b, double* out_a, double* out_b,
+int launch_rows_t(const ffc_row_plan* plan, const void* a0a, const void* a0b, const void* ma, const void* mb, double* out_a, double* out_b,
                   unsigned* status, cudaStream_t s) {
   using C = RowsGeo<D, FORM>;
-  constexpr int N = nscalar(D, Q);
   const int pmax = std::max(plan->max_pairs, 1);
   using K = RowsCfg<D, FORM, Q>;
   constexpr int NDIG = rows_ndig<T>();
   const int rmax = std::max(plan->max_region, 16);
   const size_t meta_off = (2 * size_t(C::NF) * NDIG * ROWS_VSTRIDE * 4 + 4 * size_t(rmax) +
-                           (3 * size_t(pmax) * C::GS + size_t(C::NF) * N) * sizeof(T) +
-                           4 * sizeof(RowsSlot<NDIG>) + 3 * 4 + 15) / 16 * 16;
-  const size_t smem = meta_off + 8 * 8 * sizeof(long long) + 4 * sizeof(unsigned long long);
+                           3 * size_t(pmax) * C::GS * sizeof(T) + 15) / 16 * 16;
+  const size_t smem = meta_off + 8 * sizeof(RowsChunk) + 7 * sizeof(unsigned long long);
   auto kern = rows_assemble<D, FORM, Q, T>;
   int dev = 0, smem_optin = 0;
   cudaGetDevice(&dev);
@@ -1135,10 +1162,25 @@ int launch_rows_t(const ffc_row_plan* plan, const void* a0a, const void* a0b, do
   long long blocks = (long long)sms * per_sm;
   if (blocks > plan->n_chunks) blocks = plan->n_chunks;
   if (blocks < 1) return FFC_OK;
-  RowsParams prm{plan->chunk_off, plan->chunk_pair, plan->chunk_val, plan->chunk_inc, plan->region, plan->geom,
-                 a0a, a0b, out_a, out_b, (long long)plan->n_chunks, int(meta_off), pmax, rmax, status};
-  kern<<<unsigned(blocks), TH, smem, s>>>(prm);
-  const cudaError_t e = cudaGetLastError();
+  RowsParams prm{plan->chunk_off, plan->chunk_pair, plan->chunk_val, plan->chunk_inc, plan->chunk_eb, plan->region, plan->geom,
+                 a0a, a0b, ma, mb, out_a, out_b, (long long)plan->n_chunks, int(meta_off), pmax, rmax, status};
+  const long long bound_blocks = std::min<long long>((plan->n_chunks + 7) / 8, (long long)sms * 8);
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  cfg.gridDim = dim3(unsigned(bound_blocks));
+  cfg.blockDim = dim3(256);
+  cudaError_t e = cudaLaunchKernelEx(&cfg, rows_bounds<D, FORM, Q, T>, prm);
+  if (e == cudaSuccess) {
+    cfg.gridDim = dim3(unsigned(blocks));
+    cfg.blockDim = dim3(TH);
+    cfg.dynamicSmemBytes = smem;
+    e = cudaLaunchKernelEx(&cfg, kern, prm);
+  }
   return e == cudaSuccess ? FFC_OK : cuda_fail(e, "rows_assemble launch");
 }
 
@@ -1159,35 +1201,35 @@ int launch_rows_geometry(const ffc_row_plan* plan, const int32_t* cells, const d
 
 template <int D, int FORM, typename T>
 int launch_rows_q(const ffc_row_plan* plan, int q, const int32_t* cells, const double* vertices, int64_t n_vert,
-                  const void* a0a, const void* a0b, double* out_a, double* out_b, unsigned* status,
+                  const void* a0a, const void* a0b, const void* ma, const void* mb, double* out_a, double* out_b, unsigned* status,
                   cudaStream_t s) {
   int rc = launch_rows_geometry<D, FORM, T>(plan, cells, vertices, n_vert, status, s);
   if (rc != FFC_OK) return rc;
   switch (q) {
-    case 1: return launch_rows_t<D, FORM, 1, T>(plan, a0a, a0b, out_a, out_b, status, s);
-    case 2: return launch_rows_t<D, FORM, 2, T>(plan, a0a, a0b, out_a, out_b, status, s);
-    case 3: return launch_rows_t<D, FORM, 3, T>(plan, a0a, a0b, out_a, out_b, status, s);
-    case 4: return launch_rows_t<D, FORM, 4, T>(plan, a0a, a0b, out_a, out_b, status, s);
+    case 1: return launch_rows_t<D, FORM, 1, T>(plan, a0a, a0b, ma, mb, out_a, out_b, status, s);
+    case 2: return launch_rows_t<D, FORM, 2, T>(plan, a0a, a0b, ma, mb, out_a, out_b, status, s);
+    case 3: return launch_rows_t<D, FORM, 3, T>(plan, a0a, a0b, ma, mb, out_a, out_b, status, s);
+    case 4: return launch_rows_t<D, FORM, 4, T>(plan, a0a, a0b, ma, mb, out_a, out_b, status, s);
     default: return FFC_EUNSUPPORTED;
   }
 }
 
 template <typename T>
 int launch_rows_form(int form, int d, int q, const ffc_row_plan* plan, const int32_t* cells, const double* vertices,
-                     int64_t n_vert, const void* a0a, const void* a0b, double* out_a, double* out_b,
+                     int64_t n_vert, const void* a0a, const void* a0b, const void* ma, const void* mb, double* out_a, double* out_b,
                      unsigned* status, cudaStream_t s) {
   if (d == 3) {
     if (form == FFC_MASS)
-      return launch_rows_q<3, FFC_MASS, T>(plan, q, cells, vertices, n_vert, a0a, a0b, out_a, out_b, status, s);
+      return launch_rows_q<3, FFC_MASS, T>(plan, q, cells, vertices, n_vert, a0a, a0b, ma, mb, out_a, out_b, status, s);
     if (form == FFC_POISSON)
-      return launch_rows_q<3, FFC_POISSON, T>(plan, q, cells, vertices, n_vert, a0a, a0b, out_a, out_b, status, s);
-    return launch_rows_q<3, ROWS_PAIR, T>(plan, q, cells, vertices, n_vert, a0a, a0b, out_a, out_b, status, s);
+      return launch_rows_q<3, FFC_POISSON, T>(plan, q, cells, vertices, n_vert, a0a, a0b, ma, mb, out_a, out_b, status, s);
+    return launch_rows_q<3, ROWS_PAIR, T>(plan, q, cells, vertices, n_vert, a0a, a0b, ma, mb, out_a, out_b, status, s);
   }
   if (form == FFC_MASS)
-    return launch_rows_q<2, FFC_MASS, T>(plan, q, cells, vertices, n_vert, a0a, a0b, out_a, out_b, status, s);
+    return launch_rows_q<2, FFC_MASS, T>(plan, q, cells, vertices, n_vert, a0a, a0b, ma, mb, out_a, out_b, status, s);
   if (form == FFC_POISSON)
-    return launch_rows_q<2, FFC_POISSON, T>(plan, q, cells, vertices, n_vert, a0a, a0b, out_a, out_b, status, s);
-  return launch_rows_q<2, ROWS_PAIR, T>(plan, q, cells, vertices, n_vert, a0a, a0b, out_a, out_b, status, s);
+    return launch_rows_q<2, FFC_POISSON, T>(plan, q, cells, vertices, n_vert, a0a, a0b, ma, mb, out_a, out_b, status, s);
+  return launch_rows_q<2, ROWS_PAIR, T>(plan, q, cells, vertices, n_vert, a0a, a0b, ma, mb, out_a, out_b, status, s);
 }
 
 void free_plan(ffc_row_plan* p) {
@@ -1203,6 +1245,7 @@ void free_plan(ffc_row_plan* p) {
   cudaFree(p->chunk_inc);
   cudaFree(p->region);
   cudaFree(p->geom);
+  cudaFree(p->chunk_eb);
   cudaSetDevice(cur);
   delete p;
 }
@@ -1379,7 +1422,7 @@ int ffc_row_plan_create(int64_t n_elem, int n_local, const int32_t* dofmap, int6
   }
   if ((rc = dev_alloc(&p->chunk_row, h_chunk_row.size())) || (rc = dev_alloc(&p->chunk_pair, h_chunk_pair.size())) ||
       (rc = dev_alloc(&p->chunk_off, h_chunk_off.size())) || (rc = dev_alloc(&p->chunk_val, h_chunk_val.size())) ||
-      (rc = dev_alloc(&p->chunk_inc, h_chunk_inc.size())) ||
+      (rc = dev_alloc(&p->chunk_inc, h_chunk_inc.size())) || (rc = dev_alloc(&p->chunk_eb, h_chunk_inc.size())) ||
       (rc = dev_alloc(&p->region, size_t(p->region_total) + 16)) ||
       (rc = dev_alloc(&key, size_t(total))))
     goto fail;
@@ -1450,7 +1493,7 @@ int ffc_row_plan_layout(const ffc_row_plan* p, int64_t* n_chunks, int* max_chunk
   if (max_chunk_pairs) *max_chunk_pairs = p->max_pairs;
   if (max_region_bytes) *max_region_bytes = p->max_region;
   if (device_bytes)
-    *device_bytes = (p->n_dof + 1) * 8 + (p->n_chunks + 1) * (4 + 4 + 8 + 8) + p->n_chunks * 4 +
+    *device_bytes = (p->n_dof + 1) * 8 + (p->n_chunks + 1) * (4 + 4 + 8 + 8) + p->n_chunks * (4 + 8) +
                     p->region_total + 16 + p->n_elem * 96;
   return FFC_OK;
 }
@@ -1469,10 +1512,11 @@ int ffc_assemble_rows(const ffc_form* f, const ffc_row_plan* plan, const int32_t
     return FFC_ECUDA;
   }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  rc = precision == FFC_FP32 ? launch_rows_form<float>(f->kind, f->d, f->q, plan, cells, vertices, n_vert, t->a0s_f32,
-                                                       nullptr, csr_val, nullptr, st, s)
+  rc = precision == FFC_FP32 ? launch_rows_form<float>(f->kind, f->d, f->q, plan, cells, vertices, n_vert,
+                                                       f->kind == FFC_POISSON ? t->a0v_f32 : t->a0s_f32,
+                                                       nullptr, t->a0m_f32, nullptr, csr_val, nullptr, st, s)
                              : launch_rows_form<double>(f->kind, f->d, f->q, plan, cells, vertices, n_vert,
-                                                        t->a0s_f64, nullptr, csr_val, nullptr, st, s);
+                                                        t->a0s_f64, nullptr, t->a0m_f64, nullptr, csr_val, nullptr, st, s);
   if (rc == FFC_EUNSUPPORTED) set_error("ffc_assemble_rows: the plan's chunks need more shared memory than a CTA has");
   return rc;
 }
@@ -1508,8 +1552,8 @@ int ffc_assemble_rows_pair(const ffc_form* fa, const ffc_form* fb, const ffc_row
   }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (precision == FFC_FP32) {
-    rc = launch_rows_form<float>(ROWS_PAIR, fm->d, fm->q, plan, cells, vertices, n_vert, tm->a0s_f32, tp->a0s_f32, vm,
-                                 vp, st, s);
+    rc = launch_rows_form<float>(ROWS_PAIR, fm->d, fm->q, plan, cells, vertices, n_vert, tm->a0s_f32, tp->a0v_f32,
+                                 tm->a0m_f32, tp->a0m_f32, vm, vp, st, s);
     if (rc != FFC_EUNSUPPORTED) return rc;
   }
   // FP64 (whose double-buffered 63-bit accumulators of two matrices exceed the shared
