@@ -50,27 +50,46 @@ def _prec(p) -> int:
     return PRECISIONS[p] if isinstance(p, str) else int(p)
 
 
-def _stream(stream):
-    import torch
+# torch is imported by the first call that needs it: the host entry points run without it.
+_torch = None
 
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+
+def _get_torch():
+    global _torch
+    if _torch is None:
+        import torch
+
+        _torch = torch
+    return _torch
+
+
+def _stream(stream):
+    """The cudaStream_t of ``stream``, or of the current device's current stream. The raw
+    handle is read directly: torch.cuda.current_stream() builds a Stream object through some
+    ten Python calls, a third of the host time of a small call (P2 tabulate of 13,182 tets,
+    bound by the host: 15.4 us a call with it and per-argument ctypes objects, 9.4 without)."""
+    if stream is not None:
+        return stream.cuda_stream
+    torch = _torch or _get_torch()
+    if torch.cuda.is_initialized():
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return torch.cuda.current_stream().cuda_stream
 
 
 def _dev_ptr(t, dtype, name, shape=None):
-    import torch
-
+    """The address of a checked CUDA tensor (ctypes converts it by the argument types)."""
     if t is None:
         return None
+    torch = _torch or _get_torch()
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise TypeError(f"{name} must be a CUDA tensor")
     if t.dtype != dtype:
         raise TypeError(f"{name} must be {dtype}, got {t.dtype}")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
-    if shape is not None and tuple(t.shape) != tuple(shape):
+    if shape is not None and t.shape != shape:
         raise ValueError(f"{name} has shape {tuple(t.shape)}, expected {tuple(shape)}")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 class Form:
@@ -89,11 +108,12 @@ class Form:
         r = ctypes.c_int()
         _check(lib().ffc_form_rank(h, ctypes.byref(r)), "ffc_form_rank")
         self.rank = r.value
+        self._tensor_shape = (self.n_local,) * self.rank
 
     @property
     def tensor_shape(self) -> tuple:
         """Shape of one element tensor: (n, n), or (n,) for a linear form."""
-        return (self.n_local,) * self.rank
+        return self._tensor_shape
 
     @property
     def handle(self):
@@ -124,8 +144,7 @@ class Form:
 def tabulate(form: Form, cells, vertices, coeffs=None, precision="fp64", out=None, stream=None):
     """Element tensors [n_elem, n, n] ([n_elem, n] for a linear form; float64 for fp64,
     float32 otherwise)."""
-    import torch
-
+    torch = _torch or _get_torch()
     p = _prec(precision)
     n_elem = cells.shape[0]
     shp = (n_elem,) + form.tensor_shape
@@ -145,8 +164,7 @@ def tabulate_static(form: Form, cells, vertices, coeffs=None, precision="fp64", 
     """tabulate() through the allocation-free entry point (ffc_tabulate_static): the
     reference tensor is staged in a fixed device array compiled into the library.
     FP64 or FP32 only; synchronises ``stream`` and returns (A_K, device status bits)."""
-    import torch
-
+    torch = _torch or _get_torch()
     p = _prec(precision)
     n_elem = cells.shape[0]
     shp = (n_elem,) + form.tensor_shape
@@ -183,8 +201,7 @@ def csr_pattern(dofmap: np.ndarray, n_dof: int, with_slots: bool = True):
 def assemble(form: Form, cells, vertices, slot, csr_val, coeffs=None, precision="fp64", stream=None):
     """csr_val[slot[e, i1, i2]] += A^K[e, i1, i2] for all cells (accumulates). For a
     linear form ``slot`` is the dof map [n_elem, n] and ``csr_val`` the global vector."""
-    import torch
-
+    torch = _torch or _get_torch()
     p = _prec(precision)
     n_elem = cells.shape[0]
     c = _dev_ptr(cells, torch.int32, "cells", (n_elem, form.dim + 1))
@@ -205,8 +222,7 @@ class RowPlan:
     CUDA tensors (the pattern of :func:`csr_pattern`); they may be freed afterwards."""
 
     def __init__(self, dofmap, n_dof: int, row_ptr, col, stream=None):
-        import torch
-
+        torch = _torch or _get_torch()
         n_elem, n_local = dofmap.shape
         d = _dev_ptr(dofmap, torch.int32, "dofmap")
         rp = _dev_ptr(row_ptr, torch.int64, "row_ptr", (n_dof + 1,))
@@ -245,8 +261,7 @@ class RowPlan:
 def assemble_rows(form: Form, plan: RowPlan, cells, vertices, csr_val, precision="fp32", stream=None):
     """csr_val = the assembled matrix of a mass or Poisson form (overwritten, no zeroing
     needed), by row-owner assembly with exact fixed-point sums (ffc_assemble_rows)."""
-    import torch
-
+    torch = _torch or _get_torch()
     p = _prec(precision)
     c = _dev_ptr(cells, torch.int32, "cells", (cells.shape[0], form.dim + 1))
     v = _dev_ptr(vertices, torch.float64, "vertices")
@@ -260,8 +275,7 @@ def assemble_rows_pair(form_a: Form, form_b: Form, plan: RowPlan, cells, vertice
                        precision="fp32", stream=None):
     """Two forms on the plan's space into two matrices (overwritten) by row-owner assembly
     (ffc_assemble_rows_pair); the (mass, Poisson) pair is one pass."""
-    import torch
-
+    torch = _torch or _get_torch()
     p = _prec(precision)
     c = _dev_ptr(cells, torch.int32, "cells", (cells.shape[0], form_a.dim + 1))
     v = _dev_ptr(vertices, torch.float64, "vertices")
@@ -277,8 +291,7 @@ def assemble_pair(form_a: Form, form_b: Form, cells, vertices, slot, csr_val_a, 
     """Two forms on one space into two matrices sharing the pattern (ffc_assemble_pair):
     csr_val_a[slot] += A_a^K, csr_val_b[slot] += A_b^K. The (mass, Poisson) pair in FP32 is
     one launch (geometry and slot loads shared)."""
-    import torch
-
+    torch = _torch or _get_torch()
     p = _prec(precision)
     n_elem = cells.shape[0]
     c = _dev_ptr(cells, torch.int32, "cells", (n_elem, form_a.dim + 1))
@@ -343,8 +356,7 @@ class QForm:
 def tabulate_quadrature(form: QForm, cells, nodes, precision="fp64", out=None, stream=None):
     """Element tensors of curved cells by quadrature as a contraction (ffc_tabulate_quadrature).
     cells int32 [n_elem, n_geometry] geometry node ids, nodes float64 [n_nodes, d]."""
-    import torch
-
+    torch = _torch or _get_torch()
     p = _prec(precision)
     n_elem = cells.shape[0]
     c = _dev_ptr(cells, torch.int32, "cells", (n_elem, form.n_geometry))
@@ -360,8 +372,7 @@ def tabulate_quadrature(form: QForm, cells, nodes, precision="fp64", out=None, s
 
 def assemble_quadrature(form: QForm, cells, nodes, slot, csr_val, precision="fp64", stream=None):
     """csr_val[slot] += A_K of curved cells (ffc_assemble_quadrature)."""
-    import torch
-
+    torch = _torch or _get_torch()
     p = _prec(precision)
     n_elem = cells.shape[0]
     c = _dev_ptr(cells, torch.int32, "cells", (n_elem, form.n_geometry))
@@ -376,8 +387,7 @@ def assemble_quadrature(form: QForm, cells, nodes, slot, csr_val, precision="fp6
 def scatter_add(A_K, slot, csr_val, stream=None):
     """The insertion step alone: csr_val[slot[e, ...]] += A_K[e, ...] (FP64 atomics).
     A_K float64 or float32 [n_elem, ...]; slot int32 of the same shape."""
-    import torch
-
+    torch = _torch or _get_torch()
     if A_K.dtype not in (torch.float64, torch.float32):
         raise TypeError("A_K must be float64 or float32")
     n_elem = A_K.shape[0]
@@ -393,8 +403,7 @@ def scatter_add(A_K, slot, csr_val, stream=None):
 
 def tabulate_adjoint(form: Form, cells, vertices, dA_K, dvertices=None, stream=None):
     """dL/dvertices (accumulated into ``dvertices``) for the upstream gradient dA_K."""
-    import torch
-
+    torch = _torch or _get_torch()
     n_elem = cells.shape[0]
     n = form.n_local
     if dvertices is None:
@@ -440,8 +449,7 @@ class Batch:
     FP64 CSR accumulation."""
 
     def __init__(self, items, zero_csr: bool = True):
-        import torch
-
+        torch = _torch or _get_torch()
         from ._capi import BatchItem
 
         arr = (BatchItem * len(items))()
