@@ -62,6 +62,12 @@ struct SimtCfg {
       KE_T > 0 ? KE_T : (REG_A0 ? ((R > 1 && !VEC4) ? (NA == 1 ? 16 : 32) : (NA > 1 ? 128 : 64)) : 16);
   static constexpr int KE = (KE_TARGET + EG - 1) / EG;
   static constexpr int E = EG * KE;
+  // assembly: cells ahead whose slots are asked for in L2. One thread group with one entry a
+  // thread (element tensors of 256 to 512 entries: P3 on tetrahedra) has too few loads in
+  // flight to cover HBM (178,746 tets with zeroing: Poisson FP32 462 -> 349 us, mass FP32
+  // 448 -> 324; two or four cells ahead within 1%); the others are bound by the atomics and
+  // lose 1-3% by the instruction
+  static constexpr int SLOT_AHEAD = (ASM && EG == 1 && R == 1) ? 3 : 0;
   static constexpr int NCOEF = (FORM == FFC_NS_CONVECTION) ? N : 0;
   static constexpr size_t SMEM = size_t(E) * NAP * sizeof(T) + size_t(E) * NCOEF * sizeof(double);
   // two resident CTAs per SM where the register-held reference tensor is small
@@ -245,6 +251,10 @@ __device__ __forceinline__ void simt_tile(const SimtParams& p, long long tile, u
         if constexpr (ASSEMBLE) {
           const long long en = e + C::EG;
           const bool more = (k + 1 < C::KE) && (en < p.n_elem);
+          if constexpr (C::SLOT_AHEAD > 0) {
+            if (k + C::SLOT_AHEAD < C::KE && e + C::SLOT_AHEAD * C::EG < p.n_elem && pos1[0] >= 0)
+              asm volatile("prefetch.global.L2 [%0];\n" ::"l"(p.slot + (e + C::SLOT_AHEAD * C::EG) * C::NN + pos1[0]));
+          }
 #pragma unroll
           for (int r = 0; r < C::R; ++r) {
             const bool ok = more && pos1[r] >= 0;
