@@ -216,7 +216,8 @@ def launch_list(ctx, pair_degrees, rows_degrees=()):
 
 def kernels_of(entry, precision):
     """Kernels of this library one launch-list entry starts: a row-owner call runs its
-    geometry pass and the assembly (twice for FP64, which takes the forms one at a time);
+    geometry pass and the assembly (twice for FP64, which takes the forms one at a time;
+    the small bounds pass between them is not counted);
     a fused atomic call is one kernel per launch (two for an FP64 pair)."""
     kind = entry[2]
     if kind == "rows":
@@ -295,10 +296,8 @@ def alg_bytes_tabulate(ctx, n_local, out_bytes):
 # DRAM bytes (read + write) per launch, from one `ncu` capture of the kernel on a smaller
 # mesh scaled by the cell count (positions, pairs, values and cells all grow with it); only
 # valid for the kernels as captured, other launches report null.
-# DRAM bytes per launch of the dominant kernel from an ncu capture of the current kernel
-# (scaled from a smaller mesh by the cell count); none is held for the one-digit row-owner
-# kernel, whose last capture (1.237 GB at 24^3 x 6, two-digit sums) predates it
-CAPTURED_TRAFFIC_GB = {}
+# The row-owner P4 pair: 0.221 GB read + 1.016 GB written on 24^3 x 6 cells, times 8.
+CAPTURED_TRAFFIC_GB = {("rows_mass+poisson_p4", "fp32"): 9.90}
 
 _PEAKS = {}
 
@@ -1296,9 +1295,9 @@ def measure_other(F, args, device, workload):
         clk = clocks.stop()
         assert F.status_poll() == 0
         byts = m.n_elem * (16 + 800 + 12 * 8) + m.n_vert * 24 * 2
-        # executed FP64 flops per cell: 6 symmetric combinations x 100 entries (FMA = 2),
-        # plus about 240 for J^{-1}, det J and the chain rule
-        flops = m.n_elem * (2 * 100 * 6 + 240)
+        # executed FP64 flops per cell: about 240 for J^{-1}, det J and the chain rule (the
+        # contraction runs in fixed point on the integer pipes)
+        flops = m.n_elem * 240
         cpu_rate, S = None, 0
         if not args.no_cpu_baseline:
             import multiprocessing as mp

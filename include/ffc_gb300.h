@@ -69,7 +69,10 @@ typedef enum { FFC_TRIANGLE = 2, FFC_TETRAHEDRON = 3 } ffc_cell; /* value = spat
 
 /* Arithmetic of the contraction A0 : G. J, its cofactors (adjugate) and det J are always
  * FP64: that is where a near-degenerate cell cancels. For FFC_FP64 the inverse
- * K = adj(J) / det J and G_K are FP64. For FFC_FP32 and the tensor-core precisions G_K
+ * K = adj(J) / det J and G_K are FP64, and the contraction is FP64 multiply-adds or (Poisson,
+ * the block algorithm, the adjoint) exact sums of 55- to 59-bit fixed-point products rounded
+ * once, whose error is no larger; cells whose geometry factors differ by more than the fixed
+ * point carries take the multiply-adds. For FFC_FP32 and the tensor-core precisions G_K
  * is formed in FP32, the type it is rounded to anyway (the tensor cores further split it
  * into operand parts): the dense kernels form K in FP32 from the FP64 adjugate and
  * determinant (a well-conditioned step; cells with |det J| outside [1e-30, 1e30] divide
