@@ -27,6 +27,10 @@ __device__ __forceinline__ int fix_exponent(double x) {
   return int((unsigned(__double2hiint(x)) >> 20) & 0x7ffu) - 1022;
 }
 
+// Smallest exponent of a reference-tensor row: a row of zeros takes it, so that with cell
+// exponents from -900 up the constants of the conversions below keep normal exponents.
+constexpr int FIX_ROW_MIN = -100;
+
 // x 2^(B - e) rounded to the nearest integer (halves away from zero), |x| < 2^e, 52 <= B <= 59
 template <int B>
 __device__ __forceinline__ long long fix_round(double x, int e) {

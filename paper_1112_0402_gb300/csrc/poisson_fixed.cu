@@ -134,7 +134,7 @@ __global__ void __launch_bounds__(FixedCfg<D, Q>::NT, FixedCfg<D, Q>::MIN_BLOCKS
     pos1[r] = live ? i1 * N + i1 + v : -1;
     pos2[r] = (i1 + v) * N + i1;
     double x[NP];
-    ea[r] = -1022;
+    ea[r] = FIX_ROW_MIN;
 #pragma unroll
     for (int k = 0; k < NP; ++k) {
       x[k] = live ? __ldg(p.a0t + size_t(k) * NN + pos1[r]) : 0.0;

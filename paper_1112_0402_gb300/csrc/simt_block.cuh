@@ -166,7 +166,7 @@ __device__ __forceinline__ void block_rows_init(const void* r, BlockRows<C, T>& 
       const int q = slot_of<C>(t, j);
       const int pp = q >= 0 ? pair_of_slot<C>(q) : 0;
       if constexpr (C::FIX) {
-        int e = -1022;
+        int e = FIX_ROW_MIN;
         for (int k = 0; k < C::KR; ++k) e = max(e, fix_exponent(Rg[size_t(pp) * C::KR + k]));
 #pragma unroll
         for (int k = 0; k < C::KR; ++k) b.rr[j][k] = fix_parts<C::BITS>(Rg[size_t(pp) * C::KR + k], e);
