@@ -66,7 +66,8 @@ struct SimtCfg {
   // thread (element tensors of 256 to 512 entries: P3 on tetrahedra) has too few loads in
   // flight to cover HBM (178,746 tets with zeroing: Poisson FP32 462 -> 349 us, mass FP32
   // 448 -> 324; two or four cells ahead within 1%); the others are bound by the atomics and
-  // lose 1-3% by the instruction
+  // lose 1-3% by the instruction, and so does a slot map that stays in L2: AHEAD is chosen at
+  // the launch
   static constexpr int SLOT_AHEAD = (ASM && EG == 1 && R == 1) ? 3 : 0;
   static constexpr int NCOEF = (FORM == FFC_NS_CONVECTION) ? N : 0;
   static constexpr size_t SMEM = size_t(E) * NAP * sizeof(T) + size_t(E) * NCOEF * sizeof(double);
@@ -146,7 +147,7 @@ __device__ __forceinline__ void load_a0_rows(const void* a0, int t, T (&a0r)[C::
 
 // One tile of E cells: geometry into shared memory, then contraction and store or
 // atomic scatter. Called by every thread of the block; contains block barriers.
-template <class C, int D, int FORM, int Q, typename T, bool ASSEMBLE>
+template <class C, int D, int FORM, int Q, typename T, bool ASSEMBLE, bool AHEAD = false>
 __device__ __forceinline__ void simt_tile(const SimtParams& p, long long tile, unsigned char* smem_raw,
                                           const T (&a0r)[C::REG_A0 ? C::R : 1][C::REG_A0 ? C::NA : 1]) {
   using OutT = T;
@@ -251,7 +252,7 @@ __device__ __forceinline__ void simt_tile(const SimtParams& p, long long tile, u
         if constexpr (ASSEMBLE) {
           const long long en = e + C::EG;
           const bool more = (k + 1 < C::KE) && (en < p.n_elem);
-          if constexpr (C::SLOT_AHEAD > 0) {
+          if constexpr (AHEAD) {
             if (k + C::SLOT_AHEAD < C::KE && e + C::SLOT_AHEAD * C::EG < p.n_elem && pos1[0] >= 0)
               asm volatile("prefetch.global.L2 [%0];\n" ::"l"(p.slot + (e + C::SLOT_AHEAD * C::EG) * C::NN + pos1[0]));
           }
@@ -368,7 +369,7 @@ __device__ __forceinline__ void simt_tile(const SimtParams& p, long long tile, u
   }
 }
 
-template <int D, int FORM, int Q, typename T, bool ASSEMBLE>
+template <int D, int FORM, int Q, typename T, bool ASSEMBLE, bool AHEAD = false>
 __global__ void __launch_bounds__(SimtCfg<D, FORM, Q, T, 0, 0, ASSEMBLE>::NT,
                                   SimtCfg<D, FORM, Q, T, 0, 0, ASSEMBLE>::MIN_BLOCKS)
     simt_tabulate_kernel(SimtParams p) {
@@ -378,7 +379,7 @@ __global__ void __launch_bounds__(SimtCfg<D, FORM, Q, T, 0, 0, ASSEMBLE>::NT,
   load_a0_rows<C, T>(p.a0, threadIdx.x, a0r, p.a0b);
   const long long n_tiles = (p.n_elem + C::E - 1) / C::E;
   for (long long tile = blockIdx.x; tile < n_tiles; tile += gridDim.x)
-    simt_tile<C, D, FORM, Q, T, ASSEMBLE>(p, tile, smem_raw, a0r);
+    simt_tile<C, D, FORM, Q, T, ASSEMBLE, AHEAD>(p, tile, smem_raw, a0r);
 }
 
 // Host-side launcher for one instantiation.
@@ -386,6 +387,9 @@ template <int D, int FORM, int Q, typename T, bool ASSEMBLE>
 int launch_simt_one(const SimtParams& prm, const void* a0_rows, const void* a0_cols, cudaStream_t stream) {
   using C = SimtCfg<D, FORM, Q, T, 0, 0, ASSEMBLE>;
   auto kern = simt_tabulate_kernel<D, FORM, Q, T, ASSEMBLE>;
+  // slot maps of 39 MB (24,576 P3 tets) lose 3% by asking ahead, of 77 MB (48,000) gain 35%
+  if constexpr (ASSEMBLE && C::SLOT_AHEAD > 0)
+    if (prm.n_elem * C::NN * 4 > (48ll << 20)) kern = simt_tabulate_kernel<D, FORM, Q, T, ASSEMBLE, true>;
   int sms = 0, blocks_per_sm = 1;
   if (launch_config(reinterpret_cast<const void*>(kern), C::NT, C::SMEM, -1, &sms, &blocks_per_sm) != FFC_OK)
     return FFC_ECUDA;
