@@ -27,6 +27,10 @@ __device__ __forceinline__ int fix_exponent(double x) {
   return int((unsigned(__double2hiint(x)) >> 20) & 0x7ffu) - 1022;
 }
 
+__device__ __forceinline__ bool fix_nonzero(double x) {
+  return ((unsigned(__double2hiint(x)) << 1) | unsigned(__double2loint(x))) != 0u;
+}
+
 // Smallest exponent of a reference-tensor row: a row of zeros takes it, so that with cell
 // exponents from -900 up the constants of the conversions below keep normal exponents.
 constexpr int FIX_ROW_MIN = -100;

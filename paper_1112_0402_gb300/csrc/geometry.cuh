@@ -127,18 +127,22 @@ __device__ __forceinline__ bool degenerate_test(const double J[D][D], double det
   return !(det * det > 1e-28 * h2d);
 }
 
-// Gathers the cell's vertices and computes K = J^{-1} and |det J|.
+// J of the cell, column c the edge x_{c+1} - x_0.
 template <int D>
-__device__ __forceinline__ void cell_geometry(const int32_t* __restrict__ cells, const double* __restrict__ vertices,
-                                              int64_t n_vert, int64_t e, double K[D][D], double& det_abs,
-                                              bool& degenerate, bool& bad_index) {
+__device__ __forceinline__ void cell_jacobian(const int32_t* __restrict__ cells, const double* __restrict__ vertices,
+                                              int64_t n_vert, int64_t e, double J[D][D], bool& bad_index) {
   double x[D + 1][D];
   gather_vertices<D>(cells, vertices, n_vert, e, x, bad_index);
-  double J[D][D];
 #pragma unroll
   for (int r = 0; r < D; ++r)
 #pragma unroll
     for (int c = 0; c < D; ++c) J[r][c] = x[c + 1][r] - x[0][r];
+}
+
+// K = J^{-1} and |det J|.
+template <int D>
+__device__ __forceinline__ void invert_jacobian(const double J[D][D], double K[D][D], double& det_abs,
+                                                bool& degenerate) {
   double det;
   if constexpr (D == 3) {
     const double c00 = J[1][1] * J[2][2] - J[1][2] * J[2][1];
@@ -166,6 +170,49 @@ __device__ __forceinline__ void cell_geometry(const int32_t* __restrict__ cells,
   }
   det_abs = fabs(det);
   degenerate = degenerate_test<D>(J, det);
+}
+
+// Gathers the cell's vertices and computes K = J^{-1} and |det J|.
+template <int D>
+__device__ __forceinline__ void cell_geometry(const int32_t* __restrict__ cells, const double* __restrict__ vertices,
+                                              int64_t n_vert, int64_t e, double K[D][D], double& det_abs,
+                                              bool& degenerate, bool& bad_index) {
+  double J[D][D];
+  cell_jacobian<D>(cells, vertices, n_vert, e, J, bad_index);
+  invert_jacobian<D>(J, K, det_abs, degenerate);
+}
+
+// |x| cut to FP32 in integer instructions (a conversion takes 16 clocks of the FP64 pipe a warp);
+// below FP32's normal range zero, above it infinity.
+__device__ __forceinline__ float magnitude_f32(double x) {
+  const int h = (__double2hiint(x) & 0x7fffffff) - (896 << 20);
+  return __int_as_float(min(max(h, 0), 255 << 20) << 3);
+}
+
+// The sums of magnitudes |.||.| + |.||.| behind the cofactors of J, in FP32: adj(J)[a][c], and
+// with it row a, entry c of J^{-1} times det J, errs by ulps of U[a][c], however far the two
+// products cancel.
+template <int D>
+__device__ __forceinline__ void cofactor_terms(const double J[D][D], float U[D][D]) {
+  if constexpr (D == 2) {
+    U[0][0] = magnitude_f32(J[1][1]);
+    U[0][1] = magnitude_f32(J[0][1]);
+    U[1][0] = magnitude_f32(J[1][0]);
+    U[1][1] = magnitude_f32(J[0][0]);
+  } else {
+    float A[D][D];
+#pragma unroll
+    for (int r = 0; r < D; ++r)
+#pragma unroll
+      for (int c = 0; c < D; ++c) A[r][c] = magnitude_f32(J[r][c]);
+#pragma unroll
+    for (int a = 0; a < D; ++a)
+#pragma unroll
+      for (int c = 0; c < D; ++c) {
+        const int r1 = (c + 1) % D, r2 = (c + 2) % D, c1 = (a + 1) % D, c2 = (a + 2) % D;
+        U[a][c] = fmaf(A[r1][c1], A[r2][c2], A[r1][c2] * A[r2][c1]);
+      }
+  }
 }
 
 // Geometry for an FP32 contraction: J, its cofactors (adjugate) and det J in FP64,

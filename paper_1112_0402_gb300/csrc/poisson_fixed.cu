@@ -24,11 +24,19 @@
 //             contraction) and add each value at csr_val[slot] with an FP64 atomic.
 //
 // The fixed point needs the diagonal entries of G_K within 2^6 of one another (edge-length
-// ratios up to about 8, measured by the gradients' lengths): the error, below 2^-57 of the
-// largest G_K entry times the row's largest A0 entry, is then below the rounding of FP64
-// multiply-adds on the smallest. Cells beyond that, and cells whose G_K is not finite or
-// lies outside [2^-900, 2^900], take the FP64 multiply-adds with A0 from global memory.
+// ratios up to about 8, measured by the gradients' lengths) and each off-diagonal entry either
+// zero or with terms within 2^6 of the largest entry, the terms of G_ab = det sum_c K_ac K_bc
+// taken with those of the cofactors behind K: the error, below 2^-57 of the largest G_K entry
+// times the row's largest A0 entry, is then below the rounding that an entry of G_K carries from
+// its own terms. (A tensor entry can hang on one off-diagonal entry alone. On nearly
+// axis-aligned corners, K = I plus a shear s, that is s, computed to 2^-53 s: held in units of
+// 2^-59 it would keep 27 of its bits for s = 2^-32. Cells whose rows of K cancel, jittered or
+// structured meshes among them, pass: their G_ab carries the error of the larger terms.) Other
+// cells, and cells whose G_K is not finite or lies outside [2^-900, 2^900], take the FP64
+// multiply-adds with A0 from global memory.
 #include <cuda_runtime.h>
+
+#include <cfloat>
 
 #include "ffc_internal.h"
 #include "fixed_point.cuh"
@@ -38,7 +46,8 @@
 namespace ffc {
 namespace {
 
-constexpr int FIX_BITS = 59;  // |alpha| <= 6 terms
+constexpr int FIX_BITS = 59;   // |alpha| <= 6 terms
+constexpr int FIX_SPREAD = 6;  // of a cell's G_K entries, as a power of two
 
 template <int D, int Q>
 struct FixedCfg {
@@ -88,9 +97,10 @@ constexpr int FIX_NONE = 1;
 template <int D, int Q>
 __device__ __forceinline__ void fixed_geometry(const FixedParams& p, long long e, int2* g, int* expo) {
   constexpr int NP = FixedCfg<D, Q>::NP;
-  double K[D][D], det, G[NP];
+  double J[D][D], K[D][D], det, G[NP];
   bool degenerate, bad_index;
-  cell_geometry<D>(p.cells, p.vertices, p.n_vert, e, K, det, degenerate, bad_index);
+  cell_jacobian<D>(p.cells, p.vertices, p.n_vert, e, J, bad_index);
+  invert_jacobian<D>(J, K, det, degenerate);
   geometry_tensor_k<D, FFC_POISSON, Q>(K, det, nullptr, 0.0, 0.0, [&](int a, double v) { G[a] = v; });
   if (degenerate) atomicOr(p.status, FFC_FLAG_DEGENERATE);
   if (bad_index) atomicOr(p.status, FFC_FLAG_BOUNDS);
@@ -104,7 +114,25 @@ __device__ __forceinline__ void fixed_geometry(const FixedParams& p, long long e
   int top = hi;
 #pragma unroll
   for (int a = D; a < NP; ++a) top = max(top, fix_exponent(G[a]));
-  const bool fixed = top <= 900 && lo >= -900 && hi - lo <= 6;
+  bool fixed = top <= 900 && lo >= -900 && hi - lo <= FIX_SPREAD;
+  // FP32 holds the off-diagonal entries' terms for cells of 1e-18 to 1e18; elsewhere they over-
+  // or underflow, which fails the comparison
+  float U[D][D], Ka[D][D];
+  cofactor_terms<D>(J, U);
+#pragma unroll
+  for (int a = 0; a < D; ++a)
+#pragma unroll
+    for (int c = 0; c < D; ++c) Ka[a][c] = magnitude_f32(K[a][c]);
+  const float least = top > -100 && top < 120 ? __int_as_float((top - FIX_SPREAD + 127) << 23) : INFINITY;
+#pragma unroll
+  for (int a = 0; a < D; ++a)
+#pragma unroll
+    for (int b = a + 1; b < D; ++b) {
+      float s = 0.f;
+#pragma unroll
+      for (int c = 0; c < D; ++c) s = fmaf(U[a][c], Ka[b][c], fmaf(Ka[a][c], U[b][c], s));
+      fixed = fixed && ((s >= least && s <= FLT_MAX) || !fix_nonzero(G[sym_pair_index<D>(a, b)]));
+    }
   *expo = fixed ? top * (1 << 20) : FIX_NONE;
 #pragma unroll
   for (int a = 0; a < NP; ++a)

@@ -1,0 +1,87 @@
+"""FP64 contractions in fixed point on inputs whose factors differ by many orders of magnitude:
+every entry within a few ulps of the sum of its own |terms|, as FP64 multiply-adds give it, not
+of the cell's largest.
+
+The terms run down to the products behind the cofactors: with U[a][c] the sum of the magnitudes
+of the products of cofactor (c, a) of J over |det J|, row a, entry c of K = J^-1 errs by below 8
+ulps of U (the cofactor's two products and difference 2, the determinant 4, reciprocal and
+product 2), so the terms of an entry are formed with U in the place of |K| (once in a product of
+two, the other factor K).
+
+Entries of the reference tensor that are zero but for rounding (below 2^-45 of their row's
+largest) are held to 2^-59 of that; what this changes is allowed for, entry by entry."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from synthetic import mesh as M  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+LD = np.longdouble
+ULP = 2.0 ** -53
+
+
+def _geometry(x):
+    """K, U (as above) and |det J| in extended precision, x [E, d+1, d]."""
+    J = (x[:, 1:] - x[:, :1]).transpose(0, 2, 1).astype(LD)
+    d = J.shape[1]
+    if d == 2:
+        adj = np.stack([np.stack([J[:, 1, 1], -J[:, 0, 1]], -1), np.stack([-J[:, 1, 0], J[:, 0, 0]], -1)], -2)
+        terms = np.abs(adj)
+    else:
+        adj, terms = np.empty_like(J), np.empty_like(J)
+        for a in range(3):
+            for c in range(3):
+                p = J[:, (c + 1) % 3, (a + 1) % 3] * J[:, (c + 2) % 3, (a + 2) % 3]
+                q = J[:, (c + 1) % 3, (a + 2) % 3] * J[:, (c + 2) % 3, (a + 1) % 3]
+                adj[:, a, c], terms[:, a, c] = p - q, np.abs(p) + np.abs(q)
+    det = np.einsum("ec,ec->e", adj[:, 0], J[:, :, 0])
+    return adj / det[:, None, None], terms / np.abs(det)[:, None, None], np.abs(det)
+
+
+def _corners(d, n_elem, shear, seed=3):
+    """Corner simplices J = I + lower triangle of entries of size `shear` (zero: K = I)."""
+    r = np.random.default_rng(seed)
+    J = np.eye(d) + shear * np.tril(r.uniform(0.5, 1.0, (n_elem, d, d)) * r.choice([-1, 1], (n_elem, d, d)), -1)
+    x = np.zeros((n_elem, d + 1, d))
+    x[:, 1:] = J.transpose(0, 2, 1)
+    return x
+
+
+def _on_gpu(x):
+    n, v, d = x.shape
+    ids = np.arange(n * v, dtype=np.int32).reshape(n, v)
+    return torch.as_tensor(ids, device="cuda"), torch.as_tensor(x.reshape(-1, d).copy(), device="cuda")
+
+
+def _noise(rows):
+    """2^-59 of each row's largest entry where an entry is zero but for rounding, else 0."""
+    top = np.abs(rows).max(1, keepdims=True)
+    return np.where((rows != 0) & (np.abs(rows) < 2.0 ** -45 * top), 2.0 ** -59 * top, 0.0)
+
+
+@pytest.mark.parametrize("d", [2, 3])
+@pytest.mark.parametrize("q", [1, 2, 3, 4])
+@pytest.mark.parametrize("shear", [0.0, 2.0 ** -5, 2.0 ** -7, 2.0 ** -14, 2.0 ** -27, 2.0 ** -45])
+def test_poisson_sheared_corners(d, q, shear):
+    """Off-diagonal entries of G_K far below the diagonal ones. The contraction adds at most 7
+    ulps to the 24 of G_K (two entries of K, three products and their sum, the determinant)."""
+    import paper_1112_0402_gb300 as F
+
+    form = F.Form(F.POISSON, F.TRIANGLE if d == 2 else F.TETRAHEDRON, q)
+    x = _corners(d, 101, shear)
+    A = F.tabulate(form, *_on_gpu(x)).cpu().numpy()
+    assert F.status_poll() == 0
+    K, U, det = _geometry(x)
+    n = form.n_local
+    A0 = form.reference_tensor().reshape(n, n, d, d)
+    pairs = [(a, b) for a in range(d) for b in range(a, d)]
+    A0 = np.stack([A0[:, :, a, b] + (A0[:, :, b, a] if a != b else 0.0) for a, b in pairs])
+    A0 = np.triu(A0) + np.triu(A0, 1).transpose(0, 2, 1)  # entries i1 <= i2, mirrored
+    rows = A0.reshape(len(pairs), -1).T  # [n n][pairs]
+    G = np.stack([det * (K[:, a] * K[:, b]).sum(1) for a, b in pairs], 1)
+    I = np.stack([det * (U[:, a] * np.abs(K[:, b]) + np.abs(K[:, a]) * U[:, b]).sum(1) for a, b in pairs], 1)
+    ref = (G @ rows.T.astype(LD)).reshape(A.shape)
+    tol = (I @ (32 * ULP * np.abs(rows) + _noise(rows)).T).reshape(A.shape)
+    assert (np.abs(A - ref) <= tol).all()
