@@ -31,6 +31,9 @@ __device__ __forceinline__ bool fix_nonzero(double x) {
   return ((unsigned(__double2hiint(x)) << 1) | unsigned(__double2loint(x))) != 0u;
 }
 
+// the exponent of a nonzero x, or `zero`
+__device__ __forceinline__ int fix_exponent_or(double x, int zero) { return fix_nonzero(x) ? fix_exponent(x) : zero; }
+
 // Smallest exponent of a reference-tensor row: a row of zeros takes it, so that with cell
 // exponents from -900 up the constants of the conversions below keep normal exponents.
 constexpr int FIX_ROW_MIN = -100;

@@ -22,9 +22,9 @@
 // held the FP64 pipe at 94% with the issue slots at 9%. Now the wide integer multiply-adds
 // (convection P2: 90 per value, 360 SM clocks a cell against 306 for its A_K at the HBM
 // rate), their latency at two resident CTAs and the geometry phase bound it. FP64
-// multiply-adds -> fixed point: tabulate convection P2 on 384,000 tets 2309 -> 816 us, P1
-// 240 -> 175; elasticity P3 on 48,000 tets 3180 -> 900, P2 on 162,000 2605 -> 794, P1 on
-// 384,000 1183 -> 499; assembly of 82,944 tets, convection P2 570 -> 267, elasticity P2
+// multiply-adds -> fixed point: tabulate convection P2 on 384,000 tets 2309 -> 836 us, P1
+// 237 -> 181; elasticity P3 on 48,000 tets 3180 -> 900, P2 on 162,000 2605 -> 794, P1 on
+// 384,000 1183 -> 499; assembly of 82,944 tets, convection P2 570 -> 272, elasticity P2
 // 1508 -> 477 us.
 //
 // Thread layouts. Elasticity, "row slots": a slot is (s1, c2, s2), numbered with s2
@@ -87,13 +87,17 @@ struct BlockCfg {
   // FP64 scratch per cell: J^-1, |det J| and, for elasticity, |det J| mu K K^T (symmetric)
   static constexpr int XD = D * D + 1 + (DIAG ? 0 : D * (D + 1) / 2);
   static constexpr size_t X_BYTES = FIX ? size_t(E) * (XD * sizeof(double) + 4 * sizeof(int)) : 0;
-  static constexpr size_t SMEM = G_BYTES + R_BYTES + W_BYTES + X_BYTES;
+  // FP64 convection: RowMasks and the exponents of K's entries
+  static constexpr size_t M_BYTES =
+      FIX && DIAG ? (size_t(NP2) * 16 + 4 + size_t(E) * (D * D + KR) * sizeof(int) + 15) / 16 * 16 : 0;
+  static constexpr size_t SMEM = G_BYTES + R_BYTES + W_BYTES + X_BYTES + M_BYTES;
   // register budget of the single-form FP32 kernel: two resident CTAs of 257..511 threads
   // (up to 78 registers), three of up to 256; FP64 keeps its reduced rows in registers
-  // without spills: two CTAs of up to 256 threads (convection P2 with one: 1122 against
-  // 810 us, with three and spills 986 us), one of more (elasticity P3 with two: 1262
-  // against 945 us)
-  static constexpr int MIN_BLOCKS = sizeof(T) == 8 ? (NT <= 256 ? 2 : 1) : (NT >= 512 ? 1 : (NT > 256 ? 2 : 3));
+  // without spills: three CTAs for convection P1 (two: 215 against 181 us), two of up to 256
+  // threads (convection P2 with one: 1122 against 810 us, with three and spills 986 us), one of
+  // more (elasticity P3 with two: 1262 against 945 us)
+  static constexpr int MIN_BLOCKS = sizeof(T) == 8 ? (DIAG && KR <= 12 ? 3 : (NT <= 256 ? 2 : 1))
+                                                   : (NT >= 512 ? 1 : (NT > 256 ? 2 : 3));
 };
 
 template <class C, typename T>
@@ -154,6 +158,28 @@ __device__ __forceinline__ int pair_of_slot(int q) {  // the row (s1, s2) of R a
   return s1 * C::NS + s2;
 }
 
+// Bit masks of R's rows (FP64 convection), in shared memory: bit k of `large` for the entries
+// within 2^2 of the row's largest, of `live` for the nonzero ones, and the `n_least` rows
+// `least` (both masks) whose large mask holds no other row's (P2: 22 of 100): a cell whose large
+// entries meet every one of these meets every row's.
+template <class C>
+struct RowMasks {
+  uint2* least;
+  unsigned *large, *live;
+  int* n_least;
+  int* k_expo;  // [E][D D] exponents of the cells' K, FIX_ZERO for zero
+  int* terms;   // [E][KR] exponents of det sum_c |K_ac||w_ct|
+  __device__ __forceinline__ explicit RowMasks(unsigned char* smem) {
+    least = reinterpret_cast<uint2*>(smem + C::SMEM - C::M_BYTES);
+    large = reinterpret_cast<unsigned*>(least + C::NP2);
+    live = large + C::NP2;
+    n_least = reinterpret_cast<int*>(live + C::NP2);
+    k_expo = n_least + 1;
+    terms = k_expo + C::E * (C::N / C::NS) * (C::N / C::NS);
+  }
+};
+constexpr int FIX_ZERO = -5000;  // exponent of a zero factor: below that of any product
+
 // The reduced reference tensor rows (registers, or shared memory behind the geometry
 // blocks; the first barrier of block_tile orders those stores).
 template <class C, int D, int FORM, typename T>
@@ -171,6 +197,28 @@ __device__ __forceinline__ void block_rows_init(const void* r, BlockRows<C, T>& 
 #pragma unroll
         for (int k = 0; k < C::KR; ++k) b.rr[j][k] = fix_parts<C::BITS>(Rg[size_t(pp) * C::KR + k], e);
         b.expo[j] = (e + 58 - 2 * C::BITS) * (1 << 20);
+        if constexpr (C::DIAG) {
+          static_assert(C::KR < 32 && C::NT >= C::NSL, "a bit per entry, and one to spare; a row per thread");
+          const RowMasks<C> rm(smem);
+          unsigned large = 0u, live = 0u;
+          for (int k = 0; k < C::KR; ++k) {
+            const double x = Rg[size_t(pp) * C::KR + k];
+            if (fix_exponent(x) >= e - 2) large |= 1u << k;
+            if (fix_nonzero(x)) live |= 1u << k;
+          }
+          if (t < C::NP2) {  // the first group's
+            rm.large[t] = large;
+            rm.live[t] = live;
+          }
+          if (t == 0) *rm.n_least = 0;
+          __syncthreads();
+          if (t < C::NP2) {
+            bool keep = true;
+            for (int r = 0; r < C::NP2; ++r)
+              keep = keep && ((rm.large[r] & ~large) != 0u || (rm.large[r] == large && r >= t));
+            if (keep) rm.least[atomicAdd(rm.n_least, 1)] = make_uint2(large, live);
+          }
+        }
       } else {
 #pragma unroll
         for (int k = 0; k < C::KR; ++k) b.rr[j][k] = q >= 0 ? Rg[size_t(pp) * C::KR + k] : T(0);
@@ -191,13 +239,19 @@ __device__ __forceinline__ void block_rows_init(const void* r, BlockRows<C, T>& 
 // place as fixed-point parts. (One thread per cell for all of it left five of seven warps
 // waiting: convection P2 881 against 816 us.)
 //
-// Fixed point where every row's scale is within 2^3 (convection: the rows K_a; an entry
-// errs by below 2^-53 of the smallest row's largest terms) or 2^6 (elasticity: mu (K K^T)_aa,
-// the smallest term of the blocks) of the largest one's, all finite and far from the ends
-// of the range. Other cells keep doubles and BLOCK_FIX_NONE.
+// Convection takes the fixed point where every entry of the tensor has a term R H of which R is
+// within 2^2 of its row's largest entry and H, taken as det sum_c |K_ac||w_ct|, within 2^4 of
+// the cell's largest: an entry then errs by less than FP64 multiply-adds err on the sum of its
+// |terms| (both at most 5e-16 of it). That fails for a cell whose coefficients or rows of K
+// differ by more (a component 1e-4 of the others on an aligned cell, a single nonzero node):
+// its entries that hang on the small ones would keep 58 bits less the difference. The threads
+// of each slot test their rows' masks against the cell's. An entry with no term passes (w = 0).
+// Elasticity: where mu (K K^T)_aa, the smallest term of the blocks, is within 2^6 of the
+// largest entry. All finite and far from the ends of the range. Other cells keep doubles and
+// BLOCK_FIX_NONE.
 template <class C, int D, int FORM>
 __device__ __forceinline__ void block_geometry_fixed(const SimtParams& p, long long e0, double* Gs, const double* Ws,
-                                                     double* Ks, int* Xs) {
+                                                     double* Ks, int* Xs, unsigned char* smem) {
   constexpr bool CONV = FORM == FFC_NS_CONVECTION;
   constexpr int PARTS = CONV ? C::NS : D * D;      // parts of a cell's blocks
   constexpr int PLEN = CONV ? D : C::KRP;          // stored entries of a part
@@ -205,7 +259,10 @@ __device__ __forceinline__ void block_geometry_fixed(const SimtParams& p, long l
   const int t = threadIdx.x;
   const int nc = int(p.n_elem - e0 < C::E ? p.n_elem - e0 : C::E);
   int* Ts = Xs + C::E;      // [E] largest exponent of the blocks
-  int* Ls = Xs + 2 * C::E;  // [E] smallest exponent allowed for (convection: spread of the rows)
+  int* Ls = Xs + 2 * C::E;  // [E] elasticity: smallest exponent allowed for
+  unsigned* Ms = reinterpret_cast<unsigned*>(Ls);  // [E] convection: bit k for the large entries of H
+  unsigned* Zs = Ms + C::E;                        // [E] and for the nonzero ones; bit 31: H has a denormal
+  [[maybe_unused]] const RowMasks<C> rm(smem);
   for (int el = t; el < nc; el += C::NT) {
     double K[D][D], det;
     bool degenerate, bad_index;
@@ -213,15 +270,11 @@ __device__ __forceinline__ void block_geometry_fixed(const SimtParams& p, long l
     if (degenerate) atomicOr(p.status, FFC_FLAG_DEGENERATE);
     if (bad_index) atomicOr(p.status, FFC_FLAG_BOUNDS);
     double* k = Ks + el * C::XD;
-    int lo = 1025, hi = -1022;
+    int lo = 1025;
 #pragma unroll
     for (int a = 0; a < D; ++a) {
-      int x = -1022;
 #pragma unroll
-      for (int b = 0; b < D; ++b) {
-        k[a * D + b] = K[a][b];
-        if constexpr (CONV) x = max(x, fix_exponent(K[a][b]));
-      }
+      for (int b = 0; b < D; ++b) k[a * D + b] = K[a][b];
       if constexpr (!CONV) {
 #pragma unroll
         for (int b = a; b < D; ++b) {
@@ -230,15 +283,22 @@ __device__ __forceinline__ void block_geometry_fixed(const SimtParams& p, long l
           for (int c = 0; c < D; ++c) s = fma(K[a][c], K[b][c], s);
           s *= det * p.mu;
           k[D * D + 1 + sym_pair_index<D>(a, b)] = s;
-          if (a == b) x = fix_exponent(s);
+          if (a == b) lo = min(lo, fix_exponent(s));
         }
       }
-      lo = min(lo, x);
-      hi = max(hi, x);
     }
     k[D * D] = det;
     Ts[el] = -1022;
-    Ls[el] = CONV ? hi - lo : lo;
+    if constexpr (CONV) {
+      Ms[el] = Zs[el] = 0u;
+      Xs[el] = 0;
+#pragma unroll
+      for (int a = 0; a < D; ++a)
+#pragma unroll
+        for (int b = 0; b < D; ++b) rm.k_expo[el * D * D + a * D + b] = fix_exponent_or(K[a][b], FIX_ZERO);
+    } else {
+      Ls[el] = lo;
+    }
   }
   __syncthreads();
   for (int w = t; w < nc * PARTS; w += C::NT) {
@@ -249,16 +309,29 @@ __device__ __forceinline__ void block_geometry_fixed(const SimtParams& p, long l
     int top = -1022;
     if constexpr (CONV) {
       double wc[D];
+      int we[D];
 #pragma unroll
-      for (int c = 0; c < D; ++c) wc[c] = Ws[el * C::NCOEF + c * C::NS + part];
+      for (int c = 0; c < D; ++c) {
+        wc[c] = Ws[el * C::NCOEF + c * C::NS + part];
+        we[c] = fix_exponent_or(wc[c], FIX_ZERO);
+      }
+      const int de = fix_exponent(det);
+      unsigned denormal = 0u;
 #pragma unroll
       for (int a = 0; a < D; ++a) {
         double h = 0.0;
+        int x = 2 * FIX_ZERO;
 #pragma unroll
-        for (int c = 0; c < D; ++c) h = fma(K[a * D + c], wc[c], h);
+        for (int c = 0; c < D; ++c) {
+          h = fma(K[a * D + c], wc[c], h);
+          x = max(x, rm.k_expo[el * D * D + a * D + c] + we[c]);
+        }
+        rm.terms[w * D + a] = x + de;
         g[a] = det * h;
         top = max(top, fix_exponent(g[a]));
+        if (fix_exponent(g[a]) == -1022 && fix_nonzero(g[a])) denormal = 1u << 31;
       }
+      if (denormal) atomicOr(Zs + el, denormal);
     } else {
       const int c1 = part / D, c2 = part - c1 * D;
       const double dm = det * p.mu, dl = det * p.lambda;
@@ -278,10 +351,60 @@ __device__ __forceinline__ void block_geometry_fixed(const SimtParams& p, long l
     atomicMax(Ts + el, top);
   }
   __syncthreads();
+  if constexpr (CONV) {
+    for (int w = t; w < nc * PARTS; w += C::NT) {  // the masks of the thread's parts
+      const int el = w / PARTS, part = w - el * PARTS, least = Ts[el] - 4;
+      unsigned large = 0u, live = 0u;
+#pragma unroll
+      for (int a = 0; a < D; ++a) {
+        large |= unsigned(rm.terms[w * D + a] >= least) << a;
+        live |= unsigned(rm.terms[w * D + a] > FIX_ZERO / 2) << a;
+      }
+      atomicOr(Ms + el, large << (part * D));
+      atomicOr(Zs + el, live << (part * D));
+    }
+    __syncthreads();
+    // every cell against the least masks, a lane per cell; those that miss one whose row has
+    // no term at all (few) against every row. Xs: bit 0 multiply-adds, bit 1 undecided
+    static_assert(C::NT >= C::E, "a thread or more per cell");
+    bool undecided = false;
+    const int el0 = t % C::E;
+    if (t < C::NT / C::E * C::E && el0 < nc) {
+      const unsigned large = Ms[el0], live = Zs[el0];
+      bool failed = false;
+      for (int i = t / C::E; i < *rm.n_least; i += C::NT / C::E) {
+        const uint2 r = rm.least[i];
+        if ((r.x & large) == 0u) {
+          if (r.y & live) failed = true;
+          else undecided = true;
+        }
+      }
+      if (failed || undecided) atomicOr(Xs + el0, failed ? BLOCK_FIX_NONE : 2);
+      undecided = undecided && !failed;
+    }
+    if (__syncthreads_or(undecided)) {
+      const int q = slot_of<C>(t, 0);
+      if (q >= 0) {
+        const unsigned large = rm.large[q], live = rm.live[q];
+        for (int el = t / C::NSL; el < nc; el += C::GRP)
+          if (Xs[el] == 2 && (large & Ms[el]) == 0u && (live & Zs[el]) != 0u) atomicOr(Xs + el, BLOCK_FIX_NONE);
+      }
+      __syncthreads();
+    }
+  }
   for (int w = t; w < nc * PARTS; w += C::NT) {  // each thread its own parts again
     const int el = w / PARTS, part = w - el * PARTS;
-    const int top = Ts[el], spread = CONV ? Ls[el] : top - Ls[el];
-    const bool fixed = top <= 900 && top >= -900 && spread <= (CONV ? 3 : 6);
+    int top = Ts[el];
+    bool fixed = top <= 900 && top >= -900;
+    if constexpr (CONV) {
+      if (top == -1022 && !(Zs[el] >> 31)) {  // H = 0: its parts are zero
+        fixed = true;
+        top = -900;
+      }
+      fixed = fixed && !(Xs[el] & BLOCK_FIX_NONE);
+    } else {
+      fixed = fixed && top - Ls[el] <= 6;
+    }
     if (part == 0) Xs[el] = fixed ? top * (1 << 20) : BLOCK_FIX_NONE;
     if (!fixed) continue;
     double* g = Gs + size_t(el) * C::NB * C::KRP + part * PLEN;
@@ -310,7 +433,7 @@ __device__ __forceinline__ void block_tile(const SimtParams& p, long long tile, 
   }
   __syncthreads();
   // ---- reduced geometry blocks of the tile's cells
-  if constexpr (C::FIX) block_geometry_fixed<C, D, FORM>(p, e0, Gs, Ws, Ks, Xs);
+  if constexpr (C::FIX) block_geometry_fixed<C, D, FORM>(p, e0, Gs, Ws, Ks, Xs, smem);
   else for (int el = t; el < C::E; el += C::NT) {
     const long long e = e0 + el;
     T* g = Gs + size_t(el) * C::NB * C::KRP;
@@ -390,7 +513,16 @@ __device__ __forceinline__ void block_tile(const SimtParams& p, long long tile, 
       if (eG == BLOCK_FIX_NONE) {
         const double* R = static_cast<const double*>(p.a0) + size_t(row) * C::KR;
         double acc = 0.0;
-        for (int k = 0; k < C::KR; ++k) acc = fma(gblk[k], __ldg(R + k), acc);
+        if constexpr (C::KR % 2 == 0) {  // rows of whole 16-byte pairs
+#pragma unroll 3
+          for (int k = 0; k < C::KR; k += 2) {
+            const double2 r = __ldg(reinterpret_cast<const double2*>(R + k));
+            acc = fma(gblk[k], r.x, acc);
+            acc = fma(gblk[k + 1], r.y, acc);
+          }
+        } else {
+          for (int k = 0; k < C::KR; ++k) acc = fma(gblk[k], __ldg(R + k), acc);
+        }
         return acc;
       }
       const int4* gv = reinterpret_cast<const int4*>(gblk);

@@ -85,3 +85,56 @@ def test_poisson_sheared_corners(d, q, shear):
     ref = (G @ rows.T.astype(LD)).reshape(A.shape)
     tol = (I @ (32 * ULP * np.abs(rows) + _noise(rows)).T).reshape(A.shape)
     assert (np.abs(A - ref) <= tol).all()
+
+
+def _aligned(n_elem, stretch=(1.0, 2.0, 0.5)):
+    return _corners(3, n_elem, 0.0) * np.array(stretch)
+
+
+def _jittered(n_elem):
+    m = M.unit_cube_tets(3, 0.15, 5)
+    return m.vertices[m.cells[np.arange(n_elem) % m.n_elem]]
+
+
+def _coefficients(kind, n_elem, ns):
+    r = np.random.default_rng(8)
+    w = r.standard_normal((n_elem, 3, ns))
+    if kind == "wall":  # no slip on a part of the nodes
+        return w * (r.random((n_elem, 1, ns)) < 0.5)
+    if kind == "one node":
+        return w * (np.arange(ns) == r.integers(0, ns, n_elem)[:, None])[:, None]
+    if kind == "nodes":
+        return w * np.exp2(r.uniform(-60, 0, (n_elem, 1, ns)))
+    return w * np.array(kind)[:, None]
+
+
+@pytest.mark.parametrize("q", [1, 2])
+@pytest.mark.parametrize("cells", [_aligned, _jittered])
+@pytest.mark.parametrize("kind", [(1.0, 1.0, 1.0), (1.0, 1e-4, 1.0), (1.0, 1e-8, 0.0), (1e-12, 1.0, 1e-18), "wall",
+                                  "one node", "nodes"])
+def test_convection_coefficients(q, cells, kind):
+    """Coefficients of very different size between components or nodes: a sum of at most 30
+    terms (31 ulps), each the product of K (8 ulps of U), w and |det J| (4) summed over three
+    components (4)."""
+    import paper_1112_0402_gb300 as F
+
+    form = F.Form(F.NS_CONVECTION, F.TETRAHEDRON, q)
+    n = form.n_local
+    ns, n_elem = n // 3, 131
+    x, w = cells(n_elem), _coefficients(kind, n_elem, n // 3)
+    c, v = _on_gpu(x)
+    A = F.tabulate(form, c, v, coeffs=torch.as_tensor(w.reshape(n_elem, n), device="cuda"))
+    assert F.status_poll() == 0
+    A = A.cpu().numpy().reshape(n_elem, 3, ns, 3, ns)
+    K, U, det = _geometry(x)
+    R = form.reference_tensor().reshape(n, n, n, 3)[:ns, :ns, :ns].reshape(ns * ns, ns * 3)
+    H = det[:, None, None] * np.einsum("eac,ect->eta", K, w.astype(LD))
+    T = det[:, None, None] * np.einsum("eac,ect->eta", U, np.abs(w).astype(LD))
+    ref = (H.reshape(n_elem, -1) @ R.T.astype(LD)).reshape(n_elem, ns, ns)
+    tol = 48 * ULP * (T.reshape(n_elem, -1) @ np.abs(R).T.astype(LD)).reshape(n_elem, ns, ns)
+    for i in range(3):
+        for j in range(3):
+            if i == j:
+                assert (np.abs(A[:, i, :, i] - ref) <= tol).all()
+            else:
+                assert not A[:, i, :, j].any()
