@@ -66,6 +66,25 @@ __device__ __forceinline__ int2 fix_parts(double x, int e) {
   return fix_split(fix_round<B>(x, e));
 }
 
+// The same with 29 bits more, for factors g that differ by many orders of magnitude within one
+// cell: x = (h 2^58 + m 2^29 + l) 2^(e - B - 29) cut towards zero.
+template <int B>
+__device__ __forceinline__ int4 fix_parts_wide(double x, int e) {
+  constexpr unsigned MASK = (1u << 29) - 1u;
+  const int hw = __double2hiint(x);
+  const int ex = int((unsigned(hw) >> 20) & 0x7ffu);
+  const unsigned mh = (unsigned(hw) & 0xfffffu) | (ex ? 1u << 20 : 0u);
+  const unsigned long long m = (static_cast<unsigned long long>(mh) << 32 | unsigned(__double2loint(x))) << (B - 53);
+  const int sh = e + 1022 - (ex ? ex : 1);  // >= 0
+  const long long s = hw >> 31;
+  const long long f = static_cast<long long>(m >> (sh < 63 ? sh : 63));
+  const int low = int(unsigned(sh <= 29 ? m << (29 - sh) : m >> (sh < 92 ? sh - 29 : 63)) & MASK);
+  const int2 p = fix_split((f ^ s) - s);
+  int l = (low ^ int(s)) - int(s);
+  asm("" : "+r"(l));
+  return make_int4(p.x, p.y, l, 0);
+}
+
 // The partial sums of a contraction, the middle one in two chains (a chain's latency, not
 // the multipliers, would bound a thread otherwise); `mid` starts at half a unit of the
 // final shift.
@@ -79,12 +98,36 @@ struct FixAcc {
   __device__ __forceinline__ long long sum() const { return hi + ((mid + mid2) >> 29); }
 };
 
+// The partial sums with wide factors g, in units 2^58, 2^29 and 1 of the last: five multiply-adds
+// per term, and the dropped al gl below 2^-89 of the scales. Up to 9 terms for B = 58.
+struct FixAccWide {
+  long long hi = 0, mid = 0, lo = 0;
+  __device__ __forceinline__ void add(int2 a, int4 g) {
+    hi += static_cast<long long>(a.x) * g.x;
+    mid += static_cast<long long>(a.x) * g.y;
+    mid += static_cast<long long>(a.y) * g.x;
+    lo += static_cast<long long>(a.x) * g.z;
+    lo += static_cast<long long>(a.y) * g.y;
+  }
+};
+
+// A magnitude of three words (w2 the highest, zero only for zero) rounded to a double: normalised
+// to a leading one at bit 31 of w2 and cut to 53 bits, and the next bit (halves away from zero)
+// and the exponent field `expo`, one less than that of bit 31, are added: the leading one
+// completes the field, and so does a carry of the rounding.
+__device__ __forceinline__ double fix_pack(unsigned w2, unsigned w1, unsigned w0, unsigned sign, int expo) {
+  const unsigned sh = unsigned(__clz(int(w2)));  // 32 only for zero
+  const unsigned nh = __funnelshift_l(w1, w2, sh), nl = __funnelshift_l(w0, w1, sh);
+  const unsigned up = (nl >> 10) & 1u;
+  const unsigned lo = __funnelshift_r(nl, nh, 11) + up;
+  unsigned hi = (nh >> 11) + (lo < up ? 1u : 0u) + (unsigned(expo) - (sh << 20));
+  if (w2 == 0) hi = 0;  // then lo is 0 too
+  return __hiloint2double(int(hi | sign), int(lo));
+}
+
 // v 2^ulog rounded to the nearest double, |v| < 2^63, for results with normal exponents;
 // `e20` is ulog << 20. Two forms, which a kernel can mix so that two pipes share the work.
-//
-// On the integer pipes: the magnitude is normalised to a leading one at bit 63 and cut to
-// 53 bits, and the next bit (halves away from zero) and (exponent - 1) << 52 are added: the
-// leading one completes the exponent field, and so does a carry of the rounding.
+// This one is on the integer pipes.
 __device__ __forceinline__ double fix_to_double(long long v, int e20) {
   const long long s = v >> 63;
   const unsigned long long m = static_cast<unsigned long long>((v ^ s) - s);
@@ -95,13 +138,32 @@ __device__ __forceinline__ double fix_to_double(long long v, int e20) {
     ml = 0;
     expo -= 32 << 20;
   }
-  const unsigned sh = unsigned(__clz(int(mh)));  // 32 only for zero
-  const unsigned nh = __funnelshift_l(ml, mh, sh), nl = ml << (sh & 31u);
-  const unsigned up = (nl >> 10) & 1u;
-  const unsigned lo = __funnelshift_r(nl, nh, 11) + up;
-  unsigned hi = (nh >> 11) + (lo < up ? 1u : 0u) + (unsigned(expo) - (sh << 20));
-  if (mh == 0) hi = 0;  // then lo is 0 too
-  return __hiloint2double(int(hi | (unsigned(s >> 32) & 0x80000000u)), int(lo));
+  return fix_pack(mh, ml, 0u, unsigned(s >> 32) & 0x80000000u, expo);
+}
+
+// The same for wide sums, `e20` for the unit of `hi`. A negative sum's magnitude is taken as its
+// one's complement, less by 2^-58 units.
+__device__ __forceinline__ double fix_to_double(const FixAccWide& a, int e20) {
+  constexpr long long MASK = (1ll << 29) - 1;
+  const long long mid = a.mid + (a.lo >> 29);
+  const long long v = a.hi + (mid >> 29), s = v >> 63;
+  const unsigned long long m = static_cast<unsigned long long>(v ^ s);
+  const unsigned long long f = static_cast<unsigned long long>(((mid & MASK) << 29 | (a.lo & MASK)) ^ s) << 6;
+  unsigned w2 = unsigned(m >> 32), w1 = unsigned(m), w0 = unsigned(f >> 32);
+  int expo = e20 + (1085 << 20);
+  if (m == 0) {
+    w2 = w0;
+    w1 = unsigned(f);
+    w0 = 0;
+    expo -= 64 << 20;
+  }
+  if (w2 == 0) {
+    w2 = w1;
+    w1 = w0;
+    w0 = m == 0 ? 0u : unsigned(f);
+    expo -= 32 << 20;
+  }
+  return fix_pack(w2, w1, w0, unsigned(s >> 32) & 0x80000000u, expo);
 }
 
 // On the FP64 pipe: the top 52 bits and the low 12 are placed in the significands of two

@@ -23,9 +23,10 @@
 // (convection P2: 90 per value, 360 SM clocks a cell against 306 for its A_K at the HBM
 // rate), their latency at two resident CTAs and the geometry phase bound it. FP64
 // multiply-adds -> fixed point: tabulate convection P2 on 384,000 tets 2309 -> 836 us, P1
-// 237 -> 181; elasticity P3 on 48,000 tets 3180 -> 900, P2 on 162,000 2605 -> 794, P1 on
-// 384,000 1183 -> 499; assembly of 82,944 tets, convection P2 570 -> 272, elasticity P2
-// 1508 -> 477 us.
+// 237 -> 181; elasticity, whose parts are wider (45 wide multiply-adds per value, 53 of the 69
+// SM clocks a warp's P3 values take), P3 on 48,000 tets 3183 -> 1297, P2 on 162,000 2607 -> 1221,
+// P1 on 384,000 1182 -> 630; assembly of 82,944 tets, convection P2 570 -> 272, elasticity P2
+// 1508 -> 702 us.
 //
 // Thread layouts. Elasticity, "row slots": a slot is (s1, c2, s2), numbered with s2
 // fastest, then c2, then s1, so consecutive slots are consecutive entries of element
@@ -61,7 +62,10 @@ struct BlockCfg {
   static constexpr int NN = N * N;
   static constexpr int KR = FORM == FFC_NS_CONVECTION ? NS * D : D * D;
   static constexpr int NB = FORM == FFC_NS_CONVECTION ? 1 : D * D;
-  static constexpr int VEC = 16 / int(sizeof(T));
+  // FP64 elasticity keeps its geometry entries as wide fixed-point parts, 16 bytes each
+  static constexpr bool WIDE = sizeof(T) == 8 && FORM == FFC_ELASTICITY;
+  static constexpr int GW = WIDE ? 2 : 1;  // entries of type T a geometry entry takes
+  static constexpr int VEC = WIDE ? 1 : 16 / int(sizeof(T));
   static constexpr int KRP = (KR + VEC - 1) / VEC * VEC;
   static constexpr bool DIAG = FORM == FFC_NS_CONVECTION;  // one block, on the diagonal
   static constexpr int NP2 = NS * NS;                      // pairs (s1, s2): rows of R
@@ -77,13 +81,13 @@ struct BlockCfg {
   static constexpr int E_DEF = sizeof(T) == 8 ? 64 : 128;
   static constexpr int E = KE_T > 0 ? (KE_T * GRP < 128 ? KE_T * GRP : 128) : E_DEF;  // cells per tile
   static constexpr int NCOEF = FORM == FFC_NS_CONVECTION ? N : 0;
-  static constexpr size_t G_BYTES = size_t(E) * NB * KRP * sizeof(T);
+  static constexpr size_t G_BYTES = size_t(E) * NB * KRP * GW * sizeof(T);
   static constexpr size_t R_BYTES = REG_R ? 0 : size_t(NP2) * KRP * sizeof(T);
   static constexpr size_t W_BYTES = size_t(E) * NCOEF * sizeof(double);
   // FP64 contracts in fixed point (fixed_point.cuh): the geometry blocks and the reduced
   // rows are kept as fixed-point parts, with an exponent per cell and per slot
   static constexpr bool FIX = sizeof(T) == 8;
-  static constexpr int BITS = 58;       // KR <= 31 terms
+  static constexpr int BITS = 58;       // KR <= 31 terms (wide: 9)
   // FP64 scratch per cell: J^-1, |det J| and, for elasticity, |det J| mu K K^T (symmetric)
   static constexpr int XD = D * D + 1 + (DIAG ? 0 : D * (D + 1) / 2);
   static constexpr size_t X_BYTES = FIX ? size_t(E) * (XD * sizeof(double) + 4 * sizeof(int)) : 0;
@@ -93,10 +97,11 @@ struct BlockCfg {
   static constexpr size_t SMEM = G_BYTES + R_BYTES + W_BYTES + X_BYTES + M_BYTES;
   // register budget of the single-form FP32 kernel: two resident CTAs of 257..511 threads
   // (up to 78 registers), three of up to 256; FP64 keeps its reduced rows in registers
-  // without spills: three CTAs for convection P1 (two: 215 against 181 us), two of up to 256
-  // threads (convection P2 with one: 1122 against 810 us, with three and spills 986 us), one of
-  // more (elasticity P3 with two: 1262 against 945 us)
-  static constexpr int MIN_BLOCKS = sizeof(T) == 8 ? (DIAG && KR <= 12 ? 3 : (NT <= 256 ? 2 : 1))
+  // without spills: three CTAs for convection P1 (two: 215 against 181 us), two of up to 320
+  // threads (convection P2 with one: 1122 against 810 us, with three and spills 986 us;
+  // elasticity P2 with one 1453 against 1221 us), one of more (elasticity P3 with two and
+  // narrower parts: 1262 against 945 us)
+  static constexpr int MIN_BLOCKS = sizeof(T) == 8 ? (DIAG && KR <= 12 ? 3 : (NT <= 320 ? 2 : 1))
                                                    : (NT >= 512 ? 1 : (NT > 256 ? 2 : 3));
 };
 
@@ -246,9 +251,36 @@ __device__ __forceinline__ void block_rows_init(const void* r, BlockRows<C, T>& 
 // differ by more (a component 1e-4 of the others on an aligned cell, a single nonzero node):
 // its entries that hang on the small ones would keep 58 bits less the difference. The threads
 // of each slot test their rows' masks against the cell's. An entry with no term passes (w = 0).
-// Elasticity: where mu (K K^T)_aa, the smallest term of the blocks, is within 2^6 of the
-// largest entry. All finite and far from the ends of the range. Other cells keep doubles and
-// BLOCK_FIX_NONE.
+// Elasticity: a block entry is a product of two entries of K, det and mu or lambda, and a tensor
+// entry can hang on a single one (P1: one of 9 wherever s1 and s2 are not vertex 0), on cells
+// with rows along the axes a small one. So its parts are wide, 87 bits below the cell's largest
+// entry, and the cell is taken where the product of the two smallest entries of K (those that
+// are zero but for rounding counted by the size of their cofactor's products), det and the
+// smaller of |mu| and |lambda| is within 2^28 of that.
+//
+// All finite and far from the ends of the range. Other cells keep doubles and BLOCK_FIX_NONE.
+// The exponents of the two smallest nonzero entries of K = J^-1, added. An entry below 2^-50 of
+// its cofactor's products has no digit right and counts by those.
+template <int D>
+__device__ __forceinline__ int smallest_product(const double J[D][D], const double K[D][D], double det) {
+  float U[D][D];
+  cofactor_terms<D>(J, U);
+  const float inv = 1.f / float(det);
+  int k1 = 1025, k2 = 1025;
+#pragma unroll
+  for (int a = 0; a < D; ++a)
+#pragma unroll
+    for (int c = 0; c < D; ++c) {
+      const float u = U[a][c] * inv;
+      int x = fix_exponent_or(K[a][c], 1025);
+      if (u >= 1e-30f && u <= 1e30f && magnitude_f32(K[a][c]) < u * 0x1p-50f)
+        x = int(__float_as_uint(u) >> 23) - 126;
+      k2 = min(k2, max(k1, x));
+      k1 = min(k1, x);
+    }
+  return k1 + k2;
+}
+
 template <class C, int D, int FORM>
 __device__ __forceinline__ void block_geometry_fixed(const SimtParams& p, long long e0, double* Gs, const double* Ws,
                                                      double* Ks, int* Xs, unsigned char* smem) {
@@ -256,6 +288,7 @@ __device__ __forceinline__ void block_geometry_fixed(const SimtParams& p, long l
   constexpr int PARTS = CONV ? C::NS : D * D;      // parts of a cell's blocks
   constexpr int PLEN = CONV ? D : C::KRP;          // stored entries of a part
   constexpr int PUSED = CONV ? D : D * D;          // entries used
+  constexpr int GW = C::GW;                        // doubles an entry takes
   const int t = threadIdx.x;
   const int nc = int(p.n_elem - e0 < C::E ? p.n_elem - e0 : C::E);
   int* Ts = Xs + C::E;      // [E] largest exponent of the blocks
@@ -264,13 +297,13 @@ __device__ __forceinline__ void block_geometry_fixed(const SimtParams& p, long l
   unsigned* Zs = Ms + C::E;                        // [E] and for the nonzero ones; bit 31: H has a denormal
   [[maybe_unused]] const RowMasks<C> rm(smem);
   for (int el = t; el < nc; el += C::NT) {
-    double K[D][D], det;
+    double J[D][D], K[D][D], det;
     bool degenerate, bad_index;
-    cell_geometry<D>(p.cells, p.vertices, p.n_vert, e0 + el, K, det, degenerate, bad_index);
+    cell_jacobian<D>(p.cells, p.vertices, p.n_vert, e0 + el, J, bad_index);
+    invert_jacobian<D>(J, K, det, degenerate);
     if (degenerate) atomicOr(p.status, FFC_FLAG_DEGENERATE);
     if (bad_index) atomicOr(p.status, FFC_FLAG_BOUNDS);
     double* k = Ks + el * C::XD;
-    int lo = 1025;
 #pragma unroll
     for (int a = 0; a < D; ++a) {
 #pragma unroll
@@ -281,9 +314,7 @@ __device__ __forceinline__ void block_geometry_fixed(const SimtParams& p, long l
           double s = 0.0;
 #pragma unroll
           for (int c = 0; c < D; ++c) s = fma(K[a][c], K[b][c], s);
-          s *= det * p.mu;
-          k[D * D + 1 + sym_pair_index<D>(a, b)] = s;
-          if (a == b) lo = min(lo, fix_exponent(s));
+          k[D * D + 1 + sym_pair_index<D>(a, b)] = s * (det * p.mu);
         }
       }
     }
@@ -297,7 +328,8 @@ __device__ __forceinline__ void block_geometry_fixed(const SimtParams& p, long l
 #pragma unroll
         for (int b = 0; b < D; ++b) rm.k_expo[el * D * D + a * D + b] = fix_exponent_or(K[a][b], FIX_ZERO);
     } else {
-      Ls[el] = lo;
+      Ls[el] = smallest_product<D>(J, K, det) + fix_exponent(det) +
+               min(fix_exponent_or(p.mu, 1025), fix_exponent_or(p.lambda, 1025));
     }
   }
   __syncthreads();
@@ -305,7 +337,7 @@ __device__ __forceinline__ void block_geometry_fixed(const SimtParams& p, long l
     const int el = w / PARTS, part = w - el * PARTS;
     const double* K = Ks + el * C::XD;
     const double det = K[D * D];
-    double* g = Gs + size_t(el) * C::NB * C::KRP + part * PLEN;
+    double* g = Gs + (size_t(el) * C::NB * C::KRP + part * PLEN) * GW;
     int top = -1022;
     if constexpr (CONV) {
       double wc[D];
@@ -343,7 +375,7 @@ __device__ __forceinline__ void block_geometry_fixed(const SimtParams& p, long l
           const int ab = sym_pair_index<D>(a1 < a2 ? a1 : a2, a1 < a2 ? a2 : a1);
           double v = c1 == c2 ? K[D * D + 1 + ab] : 0.0;
           v = fma(l1, K[a2 * D + c2], fma(m1, K[a2 * D + c1], v));
-          g[a1 * D + a2] = v;
+          g[(a1 * D + a2) * GW] = v;
           top = max(top, fix_exponent(v));
         }
       }
@@ -403,14 +435,16 @@ __device__ __forceinline__ void block_geometry_fixed(const SimtParams& p, long l
       }
       fixed = fixed && !(Xs[el] & BLOCK_FIX_NONE);
     } else {
-      fixed = fixed && top - Ls[el] <= 6;
+      fixed = fixed && top - Ls[el] <= 28;
     }
     if (part == 0) Xs[el] = fixed ? top * (1 << 20) : BLOCK_FIX_NONE;
     if (!fixed) continue;
-    double* g = Gs + size_t(el) * C::NB * C::KRP + part * PLEN;
-    int2* gi = reinterpret_cast<int2*>(g);
+    double* g = Gs + (size_t(el) * C::NB * C::KRP + part * PLEN) * GW;
 #pragma unroll
-    for (int k = 0; k < PUSED; ++k) gi[k] = fix_parts<C::BITS>(g[k], top);
+    for (int k = 0; k < PUSED; ++k) {
+      if constexpr (C::WIDE) reinterpret_cast<int4*>(g)[k] = fix_parts_wide<C::BITS>(g[k * GW], top);
+      else reinterpret_cast<int2*>(g)[k] = fix_parts<C::BITS>(g[k], top);
+    }
   }
 }
 
@@ -505,9 +539,8 @@ __device__ __forceinline__ void block_tile(const SimtParams& p, long long tile, 
   const int grp = C::NT >= C::NSL ? t / C::NSL : 0;
   const long long left = p.n_elem - e0;
   const int nc = int(left < C::E ? left : C::E);
-  // R[(s1,s2)] . block of cell el; `pipe`: FP64 results leave the fixed point on the FP64
-  // pipe (1) or on the integer ones (0)
-  auto contract = [&](const T* gblk, int el, int j, const T* rrow, int row, int pipe) {
+  // R[(s1,s2)] . block of cell el
+  auto contract = [&](const T* gblk, int el, int j, const T* rrow, int row) {
     if constexpr (C::FIX) {
       const int eG = Xs[el];
       if (eG == BLOCK_FIX_NONE) {
@@ -521,20 +554,27 @@ __device__ __forceinline__ void block_tile(const SimtParams& p, long long tile, 
             acc = fma(gblk[k + 1], r.y, acc);
           }
         } else {
-          for (int k = 0; k < C::KR; ++k) acc = fma(gblk[k], __ldg(R + k), acc);
+          for (int k = 0; k < C::KR; ++k) acc = fma(gblk[k * C::GW], __ldg(R + k), acc);
         }
         return acc;
       }
       const int4* gv = reinterpret_cast<const int4*>(gblk);
-      FixAcc acc;
-#pragma unroll
-      for (int k = 0; k < C::KR; k += 2) {
-        const int4 x = gv[k / 2];
-        acc.add(br.rr[j][k], make_int2(x.x, x.y));
-        if (k + 1 < C::KR) acc.add(br.rr[j][k + 1 < C::KR ? k + 1 : k], make_int2(x.z, x.w));
-      }
       const int e20 = br.expo[j] + eG;
-      return pipe ? fix_to_double_fp64(acc.sum(), e20) : fix_to_double(acc.sum(), e20);
+      if constexpr (C::WIDE) {
+        FixAccWide acc;
+#pragma unroll
+        for (int k = 0; k < C::KR; ++k) acc.add(br.rr[j][k], gv[k]);
+        return fix_to_double(acc, e20);
+      } else {
+        FixAcc acc;
+#pragma unroll
+        for (int k = 0; k < C::KR; k += 2) {
+          const int4 x = gv[k / 2];
+          acc.add(br.rr[j][k], make_int2(x.x, x.y));
+          if (k + 1 < C::KR) acc.add(br.rr[j][k + 1 < C::KR ? k + 1 : k], make_int2(x.z, x.w));
+        }
+        return fix_to_double_fp64(acc.sum(), e20);
+      }
     } else {
       const float4* gv = reinterpret_cast<const float4*>(gblk);
       T acc = T(0);
@@ -573,16 +613,17 @@ __device__ __forceinline__ void block_tile(const SimtParams& p, long long tile, 
         const int c2 = DIAG ? 0 : (q / C::NS) % D;
         const T* rrow = Rs + size_t(s1 * C::NS + s2) * C::KRP;
         for (int el = c0 + grp; el < c0 + ncc; el += C::GRP) {
-          const T* gcell = Gs + size_t(el) * C::NB * C::KRP;
+          const T* gcell = Gs + size_t(el) * C::NB * C::KRP * C::GW;
           T* cb = buf + size_t(el - c0) * C::NN;
           if constexpr (DIAG) {  // one value on the d diagonal positions
-            const T v = contract(gcell, el, j, rrow, s1 * C::NS + s2, 1);
+            const T v = contract(gcell, el, j, rrow, s1 * C::NS + s2);
 #pragma unroll
             for (int c = 0; c < D; ++c) cb[(c * C::NS + s1) * C::N + c * C::NS + s2] = v;
           } else {  // the row slot's d entries ((c1, s1), (c2, s2))
 #pragma unroll
             for (int c1 = 0; c1 < D; ++c1)
-              cb[(c1 * C::NS + s1) * C::N + c2 * C::NS + s2] = contract(gcell + (c1 * D + c2) * C::KRP, el, j, rrow, s1 * C::NS + s2, 1);
+              cb[(c1 * C::NS + s1) * C::N + c2 * C::NS + s2] =
+                  contract(gcell + (c1 * D + c2) * C::KRP * C::GW, el, j, rrow, s1 * C::NS + s2);
           }
         }
       }
@@ -639,13 +680,14 @@ __device__ __forceinline__ void block_tile(const SimtParams& p, long long tile, 
             sl_next[m] = (en < nc && live_pos[m]) ? __ldg(p.slot + (e0 + en) * C::NN + pos[m]) : -1;
           }
         }
-        const T* gcell = Gs + size_t(el) * C::NB * C::KRP;
+        const T* gcell = Gs + size_t(el) * C::NB * C::KRP * C::GW;
         T vdiag = T(0);
-        if constexpr (DIAG) vdiag = contract(gcell, el, j, rrow, s1 * C::NS + s2, 1);
+        if constexpr (DIAG) vdiag = contract(gcell, el, j, rrow, s1 * C::NS + s2);
 #pragma unroll
         for (int m = 0; m < NPOS; ++m) {
           if (ASSEMBLE && !live_pos[m]) continue;
-          const T v = DIAG ? (live_pos[m] ? vdiag : T(0)) : contract(gcell + (m * D + c2) * C::KRP, el, j, rrow, s1 * C::NS + s2, m == 0);
+          const T v = DIAG ? (live_pos[m] ? vdiag : T(0))
+                           : contract(gcell + (m * D + c2) * C::KRP * C::GW, el, j, rrow, s1 * C::NS + s2);
           if constexpr (ASSEMBLE) {
             const int sv = sl[m];
             if (sv >= 0 && sv < p.nnz) atomicAdd(p.csr_val + sv, double(v));

@@ -138,3 +138,34 @@ def test_convection_coefficients(q, cells, kind):
                 assert (np.abs(A[:, i, :, i] - ref) <= tol).all()
             else:
                 assert not A[:, i, :, j].any()
+
+
+@pytest.mark.parametrize("q", [1, 2, 3])
+@pytest.mark.parametrize("cells", [_aligned, _jittered, lambda n: _corners(3, n, 2.0 ** -12),
+                                   lambda n: _corners(3, n, 2.0 ** -27)], ids=["aligned", "jittered", "-12", "-27"])
+@pytest.mark.parametrize("lmbda", [1.25, 1e-4, 1e-8, 1e-13, 0.0, 1e4])
+def test_elasticity_small_factors(q, cells, lmbda):
+    """lambda far below mu, and entries of K far below the others: a sum of 9 terms (10 ulps),
+    each a sum of three products (3) of two entries of K (16), a Lame parameter and |det J| (6)."""
+    import paper_1112_0402_gb300 as F
+
+    form = F.Form(F.ELASTICITY, F.TETRAHEDRON, q, 1.0, lmbda)
+    n = form.n_local
+    ns, n_elem = n // 3, 67
+    x = cells(n_elem)
+    A = F.tabulate(form, *_on_gpu(x)).cpu().numpy().reshape(n_elem, 3, ns, 3, ns)
+    assert F.status_poll() == 0
+    K, U, det = _geometry(x)
+    rows = F.Form(F.POISSON, F.TETRAHEDRON, q).reference_tensor().reshape(ns * ns, 9)
+    weight, X = 40 * ULP * np.abs(rows) + _noise(rows), np.abs(K)
+    for i in range(3):
+        for j in range(3):
+            B = K[:, :, None, j] * K[:, None, :, i] + lmbda * K[:, :, None, i] * K[:, None, :, j]
+            T = (U[:, :, None, j] * X[:, None, :, i] + X[:, :, None, j] * U[:, None, :, i] +
+                 lmbda * (U[:, :, None, i] * X[:, None, :, j] + X[:, :, None, i] * U[:, None, :, j]))
+            if i == j:
+                B = B + np.einsum("eac,ebc->eab", K, K)
+                T = T + np.einsum("eac,ebc->eab", U, X) + np.einsum("eac,ebc->eab", X, U)
+            B, T = (B * det[:, None, None]).reshape(-1, 9), (T * det[:, None, None]).reshape(-1, 9)
+            err = np.abs(A[:, i, :, j].reshape(n_elem, -1) - B @ rows.T.astype(LD))
+            assert (err <= T @ weight.T).all()
