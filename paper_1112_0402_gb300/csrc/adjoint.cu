@@ -21,16 +21,28 @@
 //   load         the dA of 32/L cells at a time, asynchronously into shared memory, rows
 //                padded to an odd number of doubles;
 //   contraction  L lanes per cell: the cell's largest exponent first, then each pair i1 <= i2
-//                rounded to 55-57 bits, its two halves added as integers, times the
+//                rounded to 57 or 58 bits, its two halves added as integers, times the
 //                fixed-point A0 of the pair; the L partial sums are added as integers;
 //   chain rule   one lane per cell of the tile: FP64 J^-1, |det J| and the formula above, and
 //                FP64 atomics to the d+1 vertices.
 // Bound by the FP64 geometry and chain rule (pipe 49% busy) and the integer instructions
 // (issue 44%) at 20 resident warps. Backward pass, FP64 multiply-adds -> here: P2 on 1.05 M
-// tetrahedra 1390 -> 490 us (730-890 us with CTA-wide phases and a barrier between them),
-// P3 on 82,944 501 -> 166, P4 on 24,576 586 -> 181, P1 on 663,552 320 -> 220 us.
-// A cell whose dA is not finite or lies outside [2^-900, 2^900] takes FP64 multiply-adds
-// over all n^2 entries instead, so infinities and NaN reach the same gradients as there.
+// tetrahedra 1390 -> 510 us (730-890 us with CTA-wide phases and a barrier between them),
+// P3 on 82,944 501 -> 175, P4 on 24,576 586 -> 165, P1 on 663,552 320 -> 219 us.
+//
+// A column's sum is held in units of 2^-B of (largest A0 of the column) (largest |dA| of the
+// cell), so it keeps the digits that FP64 multiply-adds keep only while its own sum of |terms| is
+// not far below those scales: with one large dA entry on which a column does not depend, or a dA
+// of few entries, it is. The contraction therefore also sums |A0||f| of each column in half
+// precision (three packed multiply-adds beside 18 integer ones) and takes a cell only where every
+// column's sum reaches THETA; there the worst error over dA of independent, rank-one, diagonal and
+// widely spread entries is 2e-16 to 1e-15 of the sum of |terms|, as with FP64 multiply-adds (2e-16
+// to 1e-15). P1's columns have three or four terms, and 3% of the cells of a rank-one dA would fail,
+// more than half of the warps: there dA is held in wide parts (fixed_point.cuh), and a cell is
+// taken where its nonzero entries are within 2^28 of one another. Other cells, and those whose dA
+// is not finite or lies outside [2^-900, 2^900], take FP64 multiply-adds over all n^2 entries, L
+// lanes per cell.
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include "ffc_internal.h"
@@ -52,13 +64,23 @@ struct AdjCfg {
   static constexpr int STRIDE = NN | 1;  // doubles of a staged row: odd, no bank conflicts over cells
   // warps per CTA: 16 in one CTA where the reference tensor takes 30 KB (P4 tetrahedra)
   static constexpr int WARPS = NE * NP > 2000 ? 16 : 4;
-  static constexpr int MIN_BLOCKS = WARPS > 4 ? 1 : 6;
-  // bits of a factor: NE products of high parts h <= 2^(BITS - 29) are summed in 63 bits
-  static constexpr int BITS = NE > 217 ? 55 : (NE > 100 ? 56 : 57);
-  static_assert(double(NE) * double(1ull << (2 * (BITS - 29))) < 9.0e18, "the sums must fit in 63 bits");
+  static constexpr int MIN_BLOCKS = WARPS > 4 ? 1 : (NE > 200 ? 5 : 6);  // (P3 tetrahedra: 45 KB a CTA)
+  static constexpr bool WIDE = Q == 1;
+  // bits of a factor: the products of high parts h <= 2^(BITS - 29) of a lane's pairs, and of a
+  // cell's where its lanes' sums are added in one piece, stay within 63 bits
+  static constexpr int BITS = NE > 21 && NE <= 55 ? 57 : 58;
+  static constexpr bool SPLIT = NE > 55;
+  static constexpr int SUMMED = SPLIT ? (NE + L - 1) / L : NE;
+  static_assert(double(SUMMED) * double(1ull << (2 * (BITS - 29))) < 9.0e18, "the sums must fit in 63 bits");
+  // smallest sum of |A0||f| of a column, in units of 2^(its exponents): the errors of NE random
+  // roundings of 2^-BITS against 2^-53 of it
+  static constexpr int THETA = BITS - 52 - (NE > 100 ? 2 : 0) - (NE > 500 ? 2 : 0);
+  static constexpr int NH = (NP + 1) / 2;  // half2 words of a pair's |A0|
   static constexpr int ROWS = CW * STRIDE;  // doubles of a warp's staged rows
   static constexpr int WBUF = ROWS + 32 * NP;  // and its cells' sums
-  static constexpr size_t SMEM = size_t(WARPS) * WBUF * 8 + size_t(NE) * NP * 8 + size_t(NE) * 4 + size_t(NP) * 4;
+  static constexpr size_t HB = WIDE ? 0 : (size_t(NE) * NH * 4 + 7) / 8 * 8;
+  static constexpr size_t SMEM =
+      HB + size_t(WARPS) * WBUF * 8 + size_t(NE) * NP * 8 + size_t(NE) * 4 + size_t(NP) * 4;
 };
 
 // the geometry chain rule of one cell and its atomics; S = Gbar + Gbar^T
@@ -123,7 +145,8 @@ __global__ void __launch_bounds__(AdjCfg<D, Q>::WARPS * 32, AdjCfg<D, Q>::MIN_BL
   using C = AdjCfg<D, Q>;
   constexpr int N = C::N, NN = C::NN, NP = C::NP, NE = C::NE, L = C::L, NT = C::WARPS * 32;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  int2* as = reinterpret_cast<int2*>(smem_raw);                      // [NE][NP] A0, fixed point
+  __half2* ah = reinterpret_cast<__half2*>(smem_raw);                // [NE][NH] |A0| 2^-(column's exponent)
+  int2* as = reinterpret_cast<int2*>(smem_raw + C::HB);              // [NE][NP] A0, fixed point
   double* wbuf = reinterpret_cast<double*>(as + NE * NP);            // [WARPS][WBUF]
   unsigned* pairs = reinterpret_cast<unsigned*>(wbuf + C::WARPS * C::WBUF);  // [NE] positions of (i1, i2), (i2, i1)
   int* ae = reinterpret_cast<int*>(pairs + NE);                      // [NP] exponents of A0's columns
@@ -140,6 +163,14 @@ __global__ void __launch_bounds__(AdjCfg<D, Q>::WARPS * 32, AdjCfg<D, Q>::MIN_BL
   __syncthreads();
   for (int w = t; w < NE * NP; w += NT)
     as[w] = fix_parts<C::BITS>(__ldg(a0t + (w % NP) * NN + (pairs[w / NP] & 0xffffu)), ae[w % NP]);
+  if constexpr (!C::WIDE) {
+    for (int w = t; w < NE * C::NH; w += NT) {
+      const int u = w / C::NH, k = 2 * (w % C::NH), p = int(pairs[u] & 0xffffu);
+      const float x = k < NP ? float(ldexp(fabs(__ldg(a0t + k * NN + p)), -ae[k])) : 0.f;
+      const float y = k + 1 < NP ? float(ldexp(fabs(__ldg(a0t + (k + 1) * NN + p)), -ae[k + 1])) : 0.f;
+      ah[w] = __floats2half2_rn(x, y);
+    }
+  }
   __syncthreads();
   double* rows = wbuf + warp * C::WBUF;  // [CW][STRIDE] dA of the batch
   double* gp = rows + C::ROWS;           // [32][NP] Gbar + Gbar^T of the tile's cells
@@ -166,47 +197,122 @@ __global__ void __launch_bounds__(AdjCfg<D, Q>::WARPS * 32, AdjCfg<D, Q>::MIN_BL
         for (int k = l; k < NN; k += L) top = max(top, fix_exponent(x[k]));
 #pragma unroll
         for (int o = L / 2; o > 0; o >>= 1) top = max(top, __shfl_xor_sync(mask, top, o));
-        bool fixed = top <= 900 && top >= -900;
-        if (top == -1022) {  // all zero (the gradients of local functionals mostly are) or denormal
-          int any = 0;
-          for (int k = l; k < NN; k += L) any |= x[k] != 0.0;
+        double* g = gp + (b + bc) * NP;
+        bool done = false;
+        if constexpr (C::WIDE) {
+          static_assert(L == 1 && NE <= 10, "a lane has the whole cell; sums of up to 10 terms");
+          int low = 1025;  // of the nonzero entries
 #pragma unroll
-          for (int o = L / 2; o > 0; o >>= 1) any |= __shfl_xor_sync(mask, any, o);
-          fixed = any == 0;
-        }
-        if (fixed) {
-          FixAcc acc[NP];
+          for (int k = 0; k < NN; ++k) low = min(low, fix_exponent_or(x[k], 1025));
+          if (low == 1025 && top == -1022) {
+#pragma unroll
+            for (int k = 0; k < NP; ++k) g[k] = 0.0;
+            done = true;
+          } else if (top <= 900 && low >= -900 && top - low <= 28) {
+            FixAccWide acc[NP];
 #pragma unroll 2
-          for (int u = l; u < NE; u += L) {
-            const unsigned pq = pairs[u];
-            const int p1 = int(pq & 0xffffu), p2 = int(pq >> 16);
-            long long f = fix_round<C::BITS>(x[p1], top + 1);
-            if (p1 != p2) f += fix_round<C::BITS>(x[p2], top + 1);
-            const int2 g = fix_split(f);
-            const int2* a = as + u * NP;
+            for (int u = 0; u < NE; ++u) {
+              const unsigned pq = pairs[u];
+              const int p1 = int(pq & 0xffffu), p2 = int(pq >> 16);
+              int4 f = fix_parts_wide<C::BITS>(x[p1], top + 1);
+              if (p1 != p2) {
+                const int4 f2 = fix_parts_wide<C::BITS>(x[p2], top + 1);
+                f.x += f2.x, f.y += f2.y, f.z += f2.z;
+              }
+              const int2* a = as + u * NP;
 #pragma unroll
-            for (int k = 0; k < NP; ++k) acc[k].add(a[k], g);
+              for (int k = 0; k < NP; ++k) acc[k].add(a[k], f);
+            }
+#pragma unroll
+            for (int k = 0; k < NP; ++k)
+              g[k] = fix_to_double(acc[k], (ae[k] + top + 1 + 58 - 2 * C::BITS + (k < D ? 1 : 0)) * (1 << 20));
+            done = true;
+          }
+        } else {
+          if (top == -1022) {  // all zero (the gradients of local functionals mostly are) or denormal
+            int any = 0;
+            for (int k = l; k < NN; k += L) any |= x[k] != 0.0;
+#pragma unroll
+            for (int o = L / 2; o > 0; o >>= 1) any |= __shfl_xor_sync(mask, any, o);
+            if (any == 0) {
+              for (int k = l; k < NP; k += L) g[k] = 0.0;
+              done = true;
+            }
+          } else if (top <= 900 && top >= -900) {
+            FixAcc acc[NP];
+            __half2 mass[C::NH];  // sums of |A0||f| of two columns each
+#pragma unroll
+            for (int k = 0; k < C::NH; ++k) mass[k] = __float2half2_rn(0.f);
+#pragma unroll 2
+            for (int u = l; u < NE; u += L) {
+              const unsigned pq = pairs[u];
+              const int p1 = int(pq & 0xffffu), p2 = int(pq >> 16);
+              long long f = fix_round<C::BITS>(x[p1], top + 1);
+              if (p1 != p2) f += fix_round<C::BITS>(x[p2], top + 1);
+              const int2 fs = fix_split(f);
+              const int2* a = as + u * NP;
+#pragma unroll
+              for (int k = 0; k < NP; ++k) acc[k].add(a[k], fs);
+              const __half2 m = __float2half2_rn(float(abs(fs.x)) * (1.f / float(1 << (C::BITS - 29))));
+#pragma unroll
+              for (int k = 0; 2 * k < NP; ++k) mass[k] = __hfma2(ah[u * C::NH + k], m, mass[k]);
+            }
+            float least = 1.f;
+#pragma unroll
+            for (int k = 0; 2 * k < NP; ++k) {
+#pragma unroll
+              for (int o = L / 2; o > 0; o >>= 1) mass[k] = __hadd2(mass[k], __shfl_xor_sync(mask, mass[k], o));
+              const float2 m = __half22float2(mass[k]);
+              least = fminf(least, m.x);
+              if (2 * k + 1 < NP) least = fminf(least, m.y);
+            }
+            done = least >= 1.f / float(1 << C::THETA);
+            if (done) {
+#pragma unroll
+              for (int k = 0; k < NP; ++k) {
+                long long v = acc[k].sum();
+                // a diagonal entry of Gbar + Gbar^T is twice Gbar's
+                int e = ae[k] + top + 1 + 58 - 2 * C::BITS + (k < D ? 1 : 0);
+                if constexpr (C::SPLIT) {
+                  int low = int(v) & 0xfffff;
+                  v >>= 20;
+#pragma unroll
+                  for (int o = L / 2; o > 0; o >>= 1) {
+                    v += __shfl_xor_sync(mask, v, o);
+                    low += __shfl_xor_sync(mask, low, o);
+                  }
+                  v += low >> 20;
+                  low &= 0xfffff;
+                  if (v < (1ll << 42) && v >= -(1ll << 42)) {
+                    v = v * (1ll << 20) + low;
+                  } else {
+                    v = v * (1ll << 14) + (low >> 6);
+                    e += 6;
+                  }
+                } else {
+#pragma unroll
+                  for (int o = L / 2; o > 0; o >>= 1) v += __shfl_xor_sync(mask, v, o);
+                }
+                if (l == 0) g[k] = fix_to_double(v, e * (1 << 20));
+              }
+            }
+          }
+        }
+        if (!done) {  // the cell's lanes agree
+          double v[NP];
+#pragma unroll
+          for (int k = 0; k < NP; ++k) v[k] = 0.0;
+#pragma unroll 2
+          for (int i = l; i < NN; i += L) {
+#pragma unroll
+            for (int k = 0; k < NP; ++k) v[k] = fma(__ldg(a0t + k * NN + i), x[i], v[k]);
           }
 #pragma unroll
           for (int k = 0; k < NP; ++k) {
-            long long v = acc[k].sum();
 #pragma unroll
-            for (int o = L / 2; o > 0; o >>= 1) v += __shfl_xor_sync(mask, v, o);
-            // a diagonal entry of Gbar + Gbar^T is twice Gbar's
-            if (l == 0)
-              gp[(b + bc) * NP + k] =
-                  fix_to_double(v, (ae[k] + top + 1 + 58 - 2 * C::BITS + (k < D ? 1 : 0)) * (1 << 20));
+            for (int o = L / 2; o > 0; o >>= 1) v[k] += __shfl_xor_sync(mask, v[k], o);
+            if (l == 0) g[k] = k < D ? 2.0 * v[k] : v[k];
           }
-        } else if (l == 0) {
-          double g[NP];
-#pragma unroll
-          for (int k = 0; k < NP; ++k) g[k] = 0.0;
-          for (int i = 0; i < NN; ++i) {
-#pragma unroll
-            for (int k = 0; k < NP; ++k) g[k] = fma(__ldg(a0t + k * NN + i), x[i], g[k]);
-          }
-#pragma unroll
-          for (int k = 0; k < NP; ++k) gp[(b + bc) * NP + k] = k < D ? 2.0 * g[k] : g[k];
         }
       }
       __syncwarp();  // the rows are overwritten next; the sums are read below

@@ -99,7 +99,8 @@ struct FixAcc {
 };
 
 // The partial sums with wide factors g, in units 2^58, 2^29 and 1 of the last: five multiply-adds
-// per term, and the dropped al gl below 2^-89 of the scales. Up to 9 terms for B = 58.
+// per term, and the dropped al gl below 2^-89 of the scales. Up to 10 terms for B = 58, also of
+// factors g that are sums of two with half the magnitude.
 struct FixAccWide {
   long long hi = 0, mid = 0, lo = 0;
   __device__ __forceinline__ void add(int2 a, int4 g) {

@@ -169,3 +169,58 @@ def test_elasticity_small_factors(q, cells, lmbda):
             B, T = (B * det[:, None, None]).reshape(-1, 9), (T * det[:, None, None]).reshape(-1, 9)
             err = np.abs(A[:, i, :, j].reshape(n_elem, -1) - B @ rows.T.astype(LD))
             assert (err <= T @ weight.T).all()
+
+
+def _upstream(kind, form, n_elem):
+    r = np.random.default_rng(6)
+    n = form.n_local
+    x = r.standard_normal((n_elem, n, n))
+    if kind == "rank one":
+        return r.standard_normal((n_elem, n, 1)) * r.standard_normal((n_elem, 1, n))
+    if kind == "diagonal":
+        return x * np.eye(n)
+    if kind == "wide":
+        return x * np.exp2(r.uniform(-60, 0, x.shape))
+    e, i, j = np.arange(n_elem), r.integers(0, n, n_elem), r.integers(0, n, n_elem)
+    if kind == "one entry":
+        y = np.zeros_like(x)
+        y[e, i, j] = x[e, i, j]
+        return y
+    x[e, i, j] *= kind
+    return x
+
+
+@pytest.mark.parametrize("d", [2, 3])
+@pytest.mark.parametrize("q", [1, 2, 3, 4])
+@pytest.mark.parametrize("kind", ["normal", "rank one", "diagonal", "wide", "one entry", 1e6, 1e12, 1e20])
+@pytest.mark.parametrize("regular", [True, False])
+def test_adjoint_upstream_spread(d, q, kind, regular):
+    """Each component of dL/dvertices by its own terms, upstream entries of very different size.
+    Gbar is a sum of n^2 terms: roundings of at most an ulp of the sum of |terms| each, which
+    random signs add to below 2n ulps. The formula's products take two entries of K more (48
+    ulps with their sums)."""
+    import paper_1112_0402_gb300 as F
+
+    form = F.Form(F.POISSON, F.TRIANGLE if d == 2 else F.TETRAHEDRON, q)
+    n, n_elem = form.n_local, 70
+    dA = _upstream(1.0 if kind == "normal" else kind, form, n_elem)
+    if regular:
+        x = _corners(d, n_elem, 0.0)
+    else:
+        m = M.unit_square_triangles(6, 0.2, 4) if d == 2 else M.unit_cube_tets(3, 0.15, 4)
+        x = m.vertices[m.cells[np.arange(n_elem) % m.n_elem]]
+    got = F.tabulate_adjoint(form, *_on_gpu(x), torch.as_tensor(dA, device="cuda")).cpu().numpy().reshape(x.shape)
+    assert F.status_poll() == 0
+    K, U, det = _geometry(x)
+    A0 = form.reference_tensor().astype(LD)
+    G = (dA.reshape(n_elem, -1).astype(LD) @ A0).reshape(-1, d, d)
+    S = (np.abs(dA).reshape(n_elem, -1).astype(LD) @ np.abs(A0)).reshape(-1, d, d)
+
+    def gradient(G, K, sign):  # dL/dvertices; sign +1: the sum of the terms' magnitudes
+        G, KT = G + G.transpose(0, 2, 1), K.transpose(0, 2, 1)
+        c = np.einsum("eab,eak,ebk->e", G, K, K)[:, None, None] / 2
+        dJ = det[:, None, None] * (c * KT + sign * (KT @ G @ K @ KT))
+        return np.concatenate([sign * dJ.sum(2)[:, None], dJ.transpose(0, 2, 1)], 1)
+
+    tol = (2 * n + 48) * ULP * gradient(S, np.maximum(U, np.abs(K)), 1)
+    assert (np.abs(got - gradient(G, K, -1)) <= tol).all()
