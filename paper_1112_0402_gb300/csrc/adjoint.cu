@@ -74,7 +74,7 @@ struct AdjCfg {
   static_assert(double(SUMMED) * double(1ull << (2 * (BITS - 29))) < 9.0e18, "the sums must fit in 63 bits");
   // smallest sum of |A0||f| of a column, in units of 2^(its exponents): the errors of NE random
   // roundings of 2^-BITS against 2^-53 of it
-  static constexpr int THETA = BITS - 52 - (NE > 100 ? 2 : 0) - (NE > 500 ? 2 : 0);
+  [[maybe_unused]] static constexpr int THETA = BITS - 52 - (NE > 100 ? 2 : 0) - (NE > 500 ? 2 : 0);
   static constexpr int NH = (NP + 1) / 2;  // half2 words of a pair's |A0|
   static constexpr int ROWS = CW * STRIDE;  // doubles of a warp's staged rows
   static constexpr int WBUF = ROWS + 32 * NP;  // and its cells' sums

@@ -150,8 +150,8 @@ int ensure_device_tensors(ffc_form* f, DeviceTensors** out) {
       for (size_t i = 0; i < nn; ++i)
         for (size_t a = 0; a < na; ++a) padded[i * nap + a] = rows32[i * na + a];
     }
-    if ((!padded.empty() && (rc = upload(&t.a0v_f32, padded))) || (rc = upload(&t.a0s_f64, soa)) || (rc = upload(&t.a0s_f32, soa32)) || (rc = upload(&t.a0m_f64, most)) ||
-        (rc = upload(&t.a0m_f32, most32))) {
+    if ((!padded.empty() && (rc = upload(&t.a0v_f32, padded))) || (rc = upload(&t.a0s_f64, soa)) ||
+        (rc = upload(&t.a0s_f32, soa32)) || (rc = upload(&t.a0m_f64, most)) || (rc = upload(&t.a0m_f32, most32))) {
       cudaFree(t.a0_f64);
       cudaFree(t.a0t_f64);
       cudaFree(t.a0_f32);

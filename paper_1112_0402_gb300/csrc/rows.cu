@@ -327,9 +327,6 @@ __device__ __forceinline__ int bound_exponent(double b) {
   return int((static_cast<unsigned long long>(__double_as_longlong(b)) >> 52) & 0x7ffull) - 1021;
 }
 
-// 1.5 * 2^e as a float, for -126 <= e <= 127
-__device__ __forceinline__ float one_and_half_pow2(int e) { return __int_as_float(((e + 127) << 23) | (1 << 22)); }
-
 // x / 2^ulog truncated toward zero, for |x| / 2^ulog < 2^62 (integer arithmetic only)
 __device__ __forceinline__ long long to_fixed(float x, int ulog) {
   const unsigned b = __float_as_uint(x);
@@ -408,79 +405,40 @@ template <typename T>
 __host__ __device__ constexpr int rows_ndig() { return sizeof(T) == 4 ? 1 : 3; }
 
 // The digits of one contribution for |x| <= 2^(eb-1): NDIG = 3 on the grids 2^(eb-20),
-// 2^(eb-41), 2^(eb-62) (unit u = 2^(eb-62)); NDIG = 2 on the first two (u = 2^(eb-41));
-// NDIG = 1 one digit on the grid 2^(eb-31) (u = 2^(eb-31): a chunk's sums stay within
-// 2^30 u, so one 32-bit integer holds them whatever the number of contributions).
-// `magic`: the FP32 rounding constants are normal floats (-87 <= eb <= 124); otherwise
-// the integer conversion.
+// 2^(eb-41), 2^(eb-62) (unit u = 2^(eb-62)); NDIG = 1 one digit on the grid 2^(eb-31)
+// (u = 2^(eb-31): a chunk's sums stay within 2^30 u, so one 32-bit integer holds them
+// whatever the number of contributions). `magic`: the FP32 scale 2^(31 - eb) is a normal
+// float; otherwise the integer conversion.
 template <int NDIG>
 struct Digits {
-  float c1, c2, c3;
-  int b1, b2, b3, ulog;
+  static_assert(NDIG == 1 || NDIG == 3, "31 bits for FP32, 63 for FP64");
+  float scale;
+  int ulog;
   bool magic;
   __device__ __forceinline__ void init(int eb) {
-    if constexpr (NDIG == 1) {
-      // the scale 2^(31 - eb) must be a normal float
-      magic = eb >= -96 && eb <= 157;
-      c1 = __int_as_float((31 - (magic ? eb : 0) + 127) << 23);
-      c2 = c3 = 0.f;
-      b1 = b2 = b3 = 0;
-      ulog = eb - 31;
-      return;
-    }
-    magic = eb >= -87 && eb <= 124;
-    const int e = magic ? eb : 0;
-    c1 = one_and_half_pow2(e + 3);
-    c2 = one_and_half_pow2(e - 18);
-    c3 = one_and_half_pow2(e - 39);
-    b1 = __float_as_int(c1);
-    b2 = __float_as_int(c2);
-    b3 = __float_as_int(c3);
-    ulog = NDIG == 3 ? eb - 62 : eb - 41;
+    magic = NDIG == 1 && eb >= -96 && eb <= 157;
+    scale = __int_as_float((31 - (magic ? eb : 0) + 127) << 23);
+    ulog = eb - (NDIG == 1 ? 31 : 62);
   }
-  // MAGIC: the FP32 rounding constants (valid when `magic`); otherwise the integer conversion
+  // MAGIC: x 2^(31 - eb) rounded to the nearest integer (the scaling is exact; valid when
+  // `magic`); |x| <= 2^(eb-1) keeps it within 2^30. Otherwise the integer conversion
   template <bool MAGIC>
   __device__ __forceinline__ void split(float x, int (&d)[NDIG]) const {
-    if constexpr (NDIG == 1) {
-      // x 2^(31 - eb) rounded to the nearest integer (the scaling is exact); |x| <= 2^(eb-1)
-      // keeps it within 2^30
-      if constexpr (MAGIC) d[0] = __float2int_rn(x * c1);
-      else d[0] = int(to_fixed(x, ulog));
-    } else if constexpr (MAGIC) {
-      const float t1 = __fadd_rn(x, c1);
-      const float r1 = __fsub_rn(x, __fsub_rn(t1, c1));
-      const float t2 = __fadd_rn(r1, c2);
-      d[0] = __float_as_int(t1) - b1;
-      d[1] = __float_as_int(t2) - b2;
-      if constexpr (NDIG == 3) {
-        const float r2 = __fsub_rn(r1, __fsub_rn(t2, c2));
-        const float t3 = __fadd_rn(r2, c3);
-        d[2] = __float_as_int(t3) - b3;
-      }
-    } else {
-      split_int(to_fixed(x, ulog), d);
-    }
+    if constexpr (MAGIC) d[0] = __float2int_rn(x * scale);
+    else d[0] = int(to_fixed(x, ulog));
   }
   template <bool MAGIC>
   __device__ __forceinline__ void split(double x, int (&d)[NDIG]) const {
-    split_int(to_fixed(x, ulog), d);
-  }
-  __device__ __forceinline__ static void split_int(long long f, int (&d)[NDIG]) {
-    if constexpr (NDIG == 1) {
-      d[0] = int(f);
-    } else if constexpr (NDIG == 3) {
-      d[2] = int(f & 0x1FFFFFll);
-      d[1] = int((f >> 21) & 0x1FFFFFll);
-      d[0] = int(f >> 42);
-    } else {
-      d[1] = int(f & 0x1FFFFFll);
-      d[0] = int(f >> 21);
-    }
+    const long long f = to_fixed(x, ulog);
+    d[2] = int(f & 0x1FFFFFll);
+    d[1] = int((f >> 21) & 0x1FFFFFll);
+    d[0] = int(f >> 42);
   }
   // whether every nonzero one-digit result stays normal
   __device__ __forceinline__ bool stays_normal() const { return ulog >= -1022 && ulog <= 980; }
-  // a one-digit sum s * 2^ulog whose result stays normal, in 32-bit integer instructions: the magnitude is normalised to a leading one at bit 31, which
-  // completes the exponent field; exact, zero is a select
+  // a one-digit sum s * 2^ulog whose result stays normal, in 32-bit integer instructions: the
+  // magnitude is normalised to a leading one at bit 31, which completes the exponent field;
+  // exact, zero is a select
   __device__ __forceinline__ double value_int(int s) const {
     const unsigned m = unsigned(abs(s));
     unsigned sh;  // leading zeros; 2^32 - 1 for zero, whose shift gives zero
@@ -494,11 +452,10 @@ struct Digits {
   __device__ __forceinline__ double value(const int (&s)[NDIG]) const {
     if constexpr (NDIG == 1) {  // |v| < 2^31: exact in a double
       return fixed_to_double_exact(static_cast<long long>(s[0]), ulog);
-    } else if constexpr (NDIG == 3) {
-      const long long v = static_cast<long long>(s[0]) * (1ll << 42) + static_cast<long long>(s[1]) * (1ll << 21) + s[2];
+    } else {
+      const long long v =
+          static_cast<long long>(s[0]) * (1ll << 42) + static_cast<long long>(s[1]) * (1ll << 21) + s[2];
       return fixed_to_double(v, ulog);
-    } else {  // |v| < 2^52: exact in a double
-      return fixed_to_double_exact(static_cast<long long>(s[0]) * (1ll << 21) + s[1], ulog);
     }
   }
 };
@@ -518,7 +475,6 @@ template <int D, int FORM>
 struct RowsGeo {
   static constexpr int NF = FORM == ROWS_PAIR ? 2 : 1;        // matrices
   static constexpr int NP = D * (D + 1) / 2;                  // symmetric Poisson G_K entries
-  static constexpr int NAK = FORM == FFC_POISSON ? NP : 1;    // G entries of a single form
   // stored per cell: mass [|det|, |det|]; Poisson [G (NP), pad, sum|G| in slot 7]; pair [G (NP),
   // pad, |det| in slot 6, sum|G| in slot 7]
   static constexpr int GS = FORM == FFC_MASS ? 2 : 8;
@@ -526,7 +482,6 @@ struct RowsGeo {
   // G_K slots of the contribution bounds' sums: |G| of a single form, and for the pair the
   // mass's |det J| and the Poisson sum|G|, side by side for one load
   static constexpr int SUM_A = FORM == ROWS_PAIR ? DET : (FORM == FFC_POISSON ? 7 : 1);
-  static constexpr int SUM_B = 7;
 };
 
 // One thread per cell: G_K exactly as the fused CUDA-core element-tensor kernels form it
@@ -545,11 +500,11 @@ __global__ void __launch_bounds__(256) rows_geometry(const int32_t* __restrict__
 #pragma unroll
     for (int a = 0; a < C::GS; ++a) g[a] = T(0);
     bool degenerate = false, bad_index = false;
-    if constexpr (FORM == FFC_MASS || (FORM == ROWS_PAIR && sizeof(T) == 8)) {
+    if constexpr (FORM == FFC_MASS) {
       double det;
       cell_det<D>(cells, vertices, n_vert, e, det, degenerate, bad_index);
-      g[C::DET] = T(det);
-      if constexpr (FORM == FFC_MASS) g[1] = fabs(g[0]);
+      g[0] = T(det);
+      g[1] = fabs(g[0]);
     }
     if constexpr (FORM == FFC_POISSON || FORM == ROWS_PAIR) {
       bool dg, bi;
@@ -591,6 +546,14 @@ __device__ __forceinline__ void cp_async8(void* smem_dst, const void* gsrc) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 
+// Reference tensors in T, and the largest |A0| entry of each row i1 (the bounds' factor).
+struct RowsTensors {
+  const void* a;  // mass or single form (layouts: load_a0)
+  const void* b;  // pair: Poisson
+  const void* max_a;
+  const void* max_b;
+};
+
 struct RowsParams {
   const int64_t* chunk_off;
   const int32_t* chunk_pair;
@@ -599,10 +562,7 @@ struct RowsParams {
   int2* chunk_eb;  // bound exponents of the chunk's forms (ROWS_NO_BOUND: not finite)
   const unsigned char* region;
   const void* G;
-  const void* a0a;  // mass or single-form reference tensor [N][NAK][N] in T
-  const void* a0b;  // pair: the Poisson reference tensor [N][NP][N]
-  const void* ma;   // largest |A0| entry of each row i1 (the bounds' factor), of either tensor
-  const void* mb;
+  RowsTensors a0;
   double* out_a;
   double* out_b;
   long long n_chunks;
@@ -805,7 +765,7 @@ __global__ void __launch_bounds__(256) rows_bounds(RowsParams p) {
   constexpr int N = K::N, NF = C::NF;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const T big = sizeof(T) == 4 ? T(FLT_MAX) : T(DBL_MAX);
-  const T* M[2] = {static_cast<const T*>(p.ma), static_cast<const T*>(p.mb)};
+  const T* M[2] = {static_cast<const T*>(p.a0.max_a), static_cast<const T*>(p.a0.max_b)};
   grid_let_next();
   const T* G = static_cast<const T*>(p.G);
   bool waited = false;
@@ -928,8 +888,8 @@ __global__ void __launch_bounds__(sizeof(T) == 4 ? 1024 : 512, 1) rows_assemble(
   RowsChunk* ring = reinterpret_cast<RowsChunk*>(smem + p.meta_off);          // [8] chunk states
   unsigned long long* rbar = reinterpret_cast<unsigned long long*>(ring + 8);  // [4] region copies
   unsigned long long* gbar = rbar + 4;                                          // [3] geometry copies
-  const T* A0a = static_cast<const T*>(p.a0a);
-  const T* A0b = static_cast<const T*>(p.a0b);
+  const T* A0a = static_cast<const T*>(p.a0.a);
+  const T* A0b = static_cast<const T*>(p.a0.b);
   const T* Gall = static_cast<const T*>(p.G);
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   const int G1 = int(gridDim.x);
@@ -1136,8 +1096,8 @@ __global__ void __launch_bounds__(sizeof(T) == 4 ? 1024 : 512, 1) rows_assemble(
 }
 
 template <int D, int FORM, int Q, typename T>
-int launch_rows_t(const ffc_row_plan* plan, const void* a0a, const void* a0b, const void* ma, const void* mb, double* out_a, double* out_b,
-                  unsigned* status, cudaStream_t s) {
+int launch_rows_t(const ffc_row_plan* plan, const RowsTensors& a0, double* out_a, double* out_b, unsigned* status,
+                  cudaStream_t s) {
   using C = RowsGeo<D, FORM>;
   const int pmax = std::max(plan->max_pairs, 1);
   using K = RowsCfg<D, FORM, Q>;
@@ -1162,8 +1122,8 @@ int launch_rows_t(const ffc_row_plan* plan, const void* a0a, const void* a0b, co
   long long blocks = (long long)sms * per_sm;
   if (blocks > plan->n_chunks) blocks = plan->n_chunks;
   if (blocks < 1) return FFC_OK;
-  RowsParams prm{plan->chunk_off, plan->chunk_pair, plan->chunk_val, plan->chunk_inc, plan->chunk_eb, plan->region, plan->geom,
-                 a0a, a0b, ma, mb, out_a, out_b, (long long)plan->n_chunks, int(meta_off), pmax, rmax, status};
+  RowsParams prm{plan->chunk_off, plan->chunk_pair, plan->chunk_val, plan->chunk_inc, plan->chunk_eb, plan->region,
+                 plan->geom, a0, out_a, out_b, (long long)plan->n_chunks, int(meta_off), pmax, rmax, status};
   const long long bound_blocks = std::min<long long>((plan->n_chunks + 7) / 8, (long long)sms * 8);
   cudaLaunchAttribute attr{};
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1201,35 +1161,38 @@ int launch_rows_geometry(const ffc_row_plan* plan, const int32_t* cells, const d
 
 template <int D, int FORM, typename T>
 int launch_rows_q(const ffc_row_plan* plan, int q, const int32_t* cells, const double* vertices, int64_t n_vert,
-                  const void* a0a, const void* a0b, const void* ma, const void* mb, double* out_a, double* out_b, unsigned* status,
-                  cudaStream_t s) {
+                  const RowsTensors& a0, double* out_a, double* out_b, unsigned* status, cudaStream_t s) {
   int rc = launch_rows_geometry<D, FORM, T>(plan, cells, vertices, n_vert, status, s);
   if (rc != FFC_OK) return rc;
   switch (q) {
-    case 1: return launch_rows_t<D, FORM, 1, T>(plan, a0a, a0b, ma, mb, out_a, out_b, status, s);
-    case 2: return launch_rows_t<D, FORM, 2, T>(plan, a0a, a0b, ma, mb, out_a, out_b, status, s);
-    case 3: return launch_rows_t<D, FORM, 3, T>(plan, a0a, a0b, ma, mb, out_a, out_b, status, s);
-    case 4: return launch_rows_t<D, FORM, 4, T>(plan, a0a, a0b, ma, mb, out_a, out_b, status, s);
+    case 1: return launch_rows_t<D, FORM, 1, T>(plan, a0, out_a, out_b, status, s);
+    case 2: return launch_rows_t<D, FORM, 2, T>(plan, a0, out_a, out_b, status, s);
+    case 3: return launch_rows_t<D, FORM, 3, T>(plan, a0, out_a, out_b, status, s);
+    case 4: return launch_rows_t<D, FORM, 4, T>(plan, a0, out_a, out_b, status, s);
     default: return FFC_EUNSUPPORTED;
   }
 }
 
 template <typename T>
 int launch_rows_form(int form, int d, int q, const ffc_row_plan* plan, const int32_t* cells, const double* vertices,
-                     int64_t n_vert, const void* a0a, const void* a0b, const void* ma, const void* mb, double* out_a, double* out_b,
-                     unsigned* status, cudaStream_t s) {
+                     int64_t n_vert, const RowsTensors& a0, double* out_a, double* out_b, unsigned* status,
+                     cudaStream_t s) {
   if (d == 3) {
     if (form == FFC_MASS)
-      return launch_rows_q<3, FFC_MASS, T>(plan, q, cells, vertices, n_vert, a0a, a0b, ma, mb, out_a, out_b, status, s);
+      return launch_rows_q<3, FFC_MASS, T>(plan, q, cells, vertices, n_vert, a0, out_a, out_b, status, s);
     if (form == FFC_POISSON)
-      return launch_rows_q<3, FFC_POISSON, T>(plan, q, cells, vertices, n_vert, a0a, a0b, ma, mb, out_a, out_b, status, s);
-    return launch_rows_q<3, ROWS_PAIR, T>(plan, q, cells, vertices, n_vert, a0a, a0b, ma, mb, out_a, out_b, status, s);
+      return launch_rows_q<3, FFC_POISSON, T>(plan, q, cells, vertices, n_vert, a0, out_a, out_b, status, s);
+    if constexpr (sizeof(T) == 4)  // FP64 pairs are two single passes
+      return launch_rows_q<3, ROWS_PAIR, T>(plan, q, cells, vertices, n_vert, a0, out_a, out_b, status, s);
+    return FFC_EUNSUPPORTED;
   }
   if (form == FFC_MASS)
-    return launch_rows_q<2, FFC_MASS, T>(plan, q, cells, vertices, n_vert, a0a, a0b, ma, mb, out_a, out_b, status, s);
+    return launch_rows_q<2, FFC_MASS, T>(plan, q, cells, vertices, n_vert, a0, out_a, out_b, status, s);
   if (form == FFC_POISSON)
-    return launch_rows_q<2, FFC_POISSON, T>(plan, q, cells, vertices, n_vert, a0a, a0b, ma, mb, out_a, out_b, status, s);
-  return launch_rows_q<2, ROWS_PAIR, T>(plan, q, cells, vertices, n_vert, a0a, a0b, ma, mb, out_a, out_b, status, s);
+    return launch_rows_q<2, FFC_POISSON, T>(plan, q, cells, vertices, n_vert, a0, out_a, out_b, status, s);
+  if constexpr (sizeof(T) == 4)
+    return launch_rows_q<2, ROWS_PAIR, T>(plan, q, cells, vertices, n_vert, a0, out_a, out_b, status, s);
+  return FFC_EUNSUPPORTED;
 }
 
 void free_plan(ffc_row_plan* p) {
@@ -1512,11 +1475,13 @@ int ffc_assemble_rows(const ffc_form* f, const ffc_row_plan* plan, const int32_t
     return FFC_ECUDA;
   }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  rc = precision == FFC_FP32 ? launch_rows_form<float>(f->kind, f->d, f->q, plan, cells, vertices, n_vert,
-                                                       f->kind == FFC_POISSON ? t->a0v_f32 : t->a0s_f32,
-                                                       nullptr, t->a0m_f32, nullptr, csr_val, nullptr, st, s)
-                             : launch_rows_form<double>(f->kind, f->d, f->q, plan, cells, vertices, n_vert,
-                                                        t->a0s_f64, nullptr, t->a0m_f64, nullptr, csr_val, nullptr, st, s);
+  if (precision == FFC_FP32) {
+    const RowsTensors a0{f->kind == FFC_POISSON ? t->a0v_f32 : t->a0s_f32, nullptr, t->a0m_f32, nullptr};
+    rc = launch_rows_form<float>(f->kind, f->d, f->q, plan, cells, vertices, n_vert, a0, csr_val, nullptr, st, s);
+  } else {
+    const RowsTensors a0{t->a0s_f64, nullptr, t->a0m_f64, nullptr};
+    rc = launch_rows_form<double>(f->kind, f->d, f->q, plan, cells, vertices, n_vert, a0, csr_val, nullptr, st, s);
+  }
   if (rc == FFC_EUNSUPPORTED) set_error("ffc_assemble_rows: the plan's chunks need more shared memory than a CTA has");
   return rc;
 }
@@ -1552,8 +1517,8 @@ int ffc_assemble_rows_pair(const ffc_form* fa, const ffc_form* fb, const ffc_row
   }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (precision == FFC_FP32) {
-    rc = launch_rows_form<float>(ROWS_PAIR, fm->d, fm->q, plan, cells, vertices, n_vert, tm->a0s_f32, tp->a0v_f32,
-                                 tm->a0m_f32, tp->a0m_f32, vm, vp, st, s);
+    const RowsTensors a0{tm->a0s_f32, tp->a0v_f32, tm->a0m_f32, tp->a0m_f32};
+    rc = launch_rows_form<float>(ROWS_PAIR, fm->d, fm->q, plan, cells, vertices, n_vert, a0, vm, vp, st, s);
     if (rc != FFC_EUNSUPPORTED) return rc;
   }
   // FP64 (whose double-buffered 63-bit accumulators of two matrices exceed the shared

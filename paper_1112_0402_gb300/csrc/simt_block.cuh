@@ -608,23 +608,14 @@ __device__ __forceinline__ void block_tile(const SimtParams& p, long long tile, 
       for (int j = 0; j < C::PPT; ++j) {
         const int q = slot_of<C>(t, j);
         if (q < 0) continue;
-        const int s2 = q % C::NS;
-        const int s1 = DIAG ? q / C::NS : q / (C::NS * D);
-        const int c2 = DIAG ? 0 : (q / C::NS) % D;
-        const T* rrow = Rs + size_t(s1 * C::NS + s2) * C::KRP;
+        const int s2 = q % C::NS, s1 = q / C::NS;
+        const T* rrow = Rs + size_t(q) * C::KRP;
         for (int el = c0 + grp; el < c0 + ncc; el += C::GRP) {
           const T* gcell = Gs + size_t(el) * C::NB * C::KRP * C::GW;
           T* cb = buf + size_t(el - c0) * C::NN;
-          if constexpr (DIAG) {  // one value on the d diagonal positions
-            const T v = contract(gcell, el, j, rrow, s1 * C::NS + s2);
+          const T v = contract(gcell, el, j, rrow, q);  // one value on the d diagonal positions
 #pragma unroll
-            for (int c = 0; c < D; ++c) cb[(c * C::NS + s1) * C::N + c * C::NS + s2] = v;
-          } else {  // the row slot's d entries ((c1, s1), (c2, s2))
-#pragma unroll
-            for (int c1 = 0; c1 < D; ++c1)
-              cb[(c1 * C::NS + s1) * C::N + c2 * C::NS + s2] =
-                  contract(gcell + (c1 * D + c2) * C::KRP * C::GW, el, j, rrow, s1 * C::NS + s2);
-          }
+          for (int c = 0; c < D; ++c) cb[(c * C::NS + s1) * C::N + c * C::NS + s2] = v;
         }
       }
       fence_async_smem();
