@@ -304,7 +304,7 @@ void ffc_batch_destroy(ffc_batch* b);
  * e * n_local + i1, the groups' extents, and for every pair and local
  * column i2 the position of column dofmap[e][i2] inside the chunk (uint16). It owns
  * about n_elem * n_local * (2 * n_local + 4) + n_dof * 8 bytes of device memory plus an
- * [n_elem][12]-double geometry scratch (ffc_row_plan_layout reports the exact figure);
+ * [n_elem][8]-double geometry scratch (ffc_row_plan_layout reports the exact figure);
  * row_ptr is copied, so dofmap, row_ptr and col may be freed afterwards. The call
  * synchronises `stream`.
  * Errors: FFC_EBOUNDS for a dof id outside [0, n_dof) or a (row, col) pair of a cell

@@ -68,6 +68,7 @@ constexpr int ROWS_VSTRIDE = ROWS_VMAX + 4;  // ints of one digit array: a chunk
 constexpr int ROWS_PMAX = 320;            // pairs of one chunk (a multiple of 32)
 constexpr int ROWS_MAX_INCIDENCE = 1023;  // digit sums of 21-bit digits stay within 32 bits
 constexpr int ROWS_MAX_LOCAL = 64;        // local dofs per cell the plan carries
+constexpr int ROWS_GEOM = 8;              // doubles of geometry scratch per cell (RowsGeo::GS, FP64)
 
 constexpr int ROWS_WARPS = 32;            // equal shares of a chunk's pairs the plan prepares
 
@@ -109,7 +110,7 @@ struct ffc_row_plan {
   int64_t* chunk_val = nullptr;     // [n_chunks + 1] first CSR value of each chunk
   int32_t* chunk_inc = nullptr;     // [n_chunks] most pairs of one row in the chunk
   unsigned char* region = nullptr;  // [region_total] chunk regions (see region_bytes)
-  void* geom = nullptr;             // per-cell geometry scratch, [n_elem][12] doubles
+  void* geom = nullptr;             // per-cell geometry scratch, [n_elem][ROWS_GEOM] doubles
   int2* chunk_eb = nullptr;         // [n_chunks] scratch: the chunk's bound exponents (two forms)
 };
 
@@ -478,6 +479,7 @@ struct RowsGeo {
   // stored per cell: mass [|det|, |det|]; Poisson [G (NP), pad, sum|G| in slot 7]; pair [G (NP),
   // pad, |det| in slot 6, sum|G| in slot 7]
   static constexpr int GS = FORM == FFC_MASS ? 2 : 8;
+  static_assert(GS <= ROWS_GEOM, "the plan's scratch");
   static constexpr int DET = FORM == ROWS_PAIR ? 6 : 0;
   // G_K slots of the contribution bounds' sums: |G| of a single form, and for the pair the
   // mass's |det J| and the Poisson sum|G|, side by side for one load
@@ -1299,7 +1301,7 @@ int ffc_row_plan_create(int64_t n_elem, int n_local, const int32_t* dofmap, int6
   if ((rc = dev_alloc(&p->row_ptr, size_t(n_dof) + 1)) || (rc = dev_alloc(&inc_ptr, size_t(n_dof) + 1)) ||
       (rc = dev_alloc(&inc_tmp, size_t(total))) || (rc = dev_alloc(&fill, size_t(n_dof))) ||
       (rc = dev_alloc(&sums, size_t(nb))) || (rc = dev_alloc(&err, 1)) ||
-      (rc = dev_alloc(reinterpret_cast<double**>(&p->geom), size_t(n_elem) * 12)))
+      (rc = dev_alloc(reinterpret_cast<double**>(&p->geom), size_t(n_elem) * ROWS_GEOM)))
     goto fail;
   if ((e = cudaMemcpyAsync(p->row_ptr, row_ptr, (size_t(n_dof) + 1) * sizeof(int64_t), cudaMemcpyDeviceToDevice,
                            s)) != cudaSuccess ||
@@ -1457,7 +1459,7 @@ int ffc_row_plan_layout(const ffc_row_plan* p, int64_t* n_chunks, int* max_chunk
   if (max_region_bytes) *max_region_bytes = p->max_region;
   if (device_bytes)
     *device_bytes = (p->n_dof + 1) * 8 + (p->n_chunks + 1) * (4 + 4 + 8 + 8) + p->n_chunks * (4 + 8) +
-                    p->region_total + 16 + p->n_elem * 96;
+                    p->region_total + 16 + p->n_elem * ROWS_GEOM * 8;
   return FFC_OK;
 }
 
