@@ -66,8 +66,8 @@ struct SimtCfg {
   // thread (element tensors of 256 to 512 entries: P3 on tetrahedra) has too few loads in
   // flight to cover HBM (178,746 tets with zeroing: Poisson FP32 462 -> 349 us, mass FP32
   // 448 -> 324; two or four cells ahead within 1%); the others are bound by the atomics and
-  // lose 1-3% by the instruction, and so does a slot map that stays in L2: AHEAD is chosen at
-  // the launch
+  // lose 1-3% by the instruction, and so does a small slot map that stays in L2 from one call to
+  // the next: AHEAD is chosen at the launch
   static constexpr int SLOT_AHEAD = (ASM && EG == 1 && R == 1) ? 3 : 0;
   static constexpr int NCOEF = (FORM == FFC_NS_CONVECTION) ? N : 0;
   static constexpr size_t SMEM = size_t(E) * NAP * sizeof(T) + size_t(E) * NCOEF * sizeof(double);
@@ -387,9 +387,13 @@ template <int D, int FORM, int Q, typename T, bool ASSEMBLE>
 int launch_simt_one(const SimtParams& prm, const void* a0_rows, const void* a0_cols, cudaStream_t stream) {
   using C = SimtCfg<D, FORM, Q, T, 0, 0, ASSEMBLE>;
   auto kern = simt_tabulate_kernel<D, FORM, Q, T, ASSEMBLE>;
-  // slot maps of 39 MB (24,576 P3 tets) lose 3% by asking ahead, of 77 MB (48,000) gain 35%
+  // The slots ahead are asked for above 32 MB of slot map, which with the values (their loads
+  // and atomics) is what a repeated call still finds in L2. Without -> with, repeated calls /
+  // after the L2 was overwritten, P3 mass FP32 with zeroing: 25 MB 32 -> 35 / 47 -> 38 us, 38 MB
+  // 54 -> 46 / 85 -> 45, 45 MB 81 -> 68 / 88 -> 70, 73 MB 135 -> 90, 273 MB 449 -> 323; Poisson
+  // 25 MB 53 -> 53 / 84 -> 61, 38 MB 61 -> 60 / 89 -> 68, 45 MB 88 -> 70, 273 MB 463 -> 350
   if constexpr (ASSEMBLE && C::SLOT_AHEAD > 0)
-    if (prm.n_elem * C::NN * 4 > (48ll << 20)) kern = simt_tabulate_kernel<D, FORM, Q, T, ASSEMBLE, true>;
+    if (prm.n_elem * C::NN * 4 > (32ll << 20)) kern = simt_tabulate_kernel<D, FORM, Q, T, ASSEMBLE, true>;
   int sms = 0, blocks_per_sm = 1;
   if (launch_config(reinterpret_cast<const void*>(kern), C::NT, C::SMEM, -1, &sms, &blocks_per_sm) != FFC_OK)
     return FFC_ECUDA;
