@@ -72,7 +72,10 @@ def _stream(stream):
         return stream.cuda_stream
     torch = _torch or _get_torch()
     if torch.cuda.is_initialized():
-        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+        try:  # private entry points: a release without them takes the public call
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+        except AttributeError:
+            pass
     return torch.cuda.current_stream().cuda_stream
 
 
