@@ -1,5 +1,12 @@
 """The benchmark's count of the kernels it starts."""
-import bench
+import os
+import sys
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+if ROOT not in sys.path:
+    sys.path.insert(0, ROOT)
+
+import bench  # noqa: E402
 
 
 def test_a_row_owner_pass_is_three_launches():
