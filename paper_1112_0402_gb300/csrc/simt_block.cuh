@@ -245,9 +245,10 @@ __device__ __forceinline__ void block_rows_init(const void* r, BlockRows<C, T>& 
 // waiting: convection P2 881 against 816 us.)
 //
 // Convection takes the fixed point where every entry of the tensor has a term R H of which R is
-// within 2^2 of its row's largest entry and H, taken as det sum_c |K_ac||w_ct|, within 2^4 of
-// the cell's largest: an entry then errs by less than FP64 multiply-adds err on the sum of its
-// |terms| (both at most 5e-16 of it). That fails for a cell whose coefficients or rows of K
+// within 2^2 of its row's largest entry and H, taken as det sum_c |K_ac||w_ct|, within 2^3 of
+// the cell's largest: an entry then errs by no more of the sum of its |terms| than FP64
+// multiply-adds (worst of random, aligned, stretched, one-sided and widely spread inputs 5.4e-16
+// against 5.0e-16 for P1, 4.3e-16 against 1.0e-15 for P2; with 2^4 1.7e-15). That fails for a cell whose coefficients or rows of K
 // differ by more (a component 1e-4 of the others on an aligned cell, a single nonzero node):
 // its entries that hang on the small ones would keep 58 bits less the difference. The threads
 // of each slot test their rows' masks against the cell's. An entry with no term passes (w = 0).
@@ -385,7 +386,7 @@ __device__ __forceinline__ void block_geometry_fixed(const SimtParams& p, long l
   __syncthreads();
   if constexpr (CONV) {
     for (int w = t; w < nc * PARTS; w += C::NT) {  // the masks of the thread's parts
-      const int el = w / PARTS, part = w - el * PARTS, least = Ts[el] - 4;
+      const int el = w / PARTS, part = w - el * PARTS, least = Ts[el] - 3;
       unsigned large = 0u, live = 0u;
 #pragma unroll
       for (int a = 0; a < D; ++a) {
