@@ -70,9 +70,12 @@ typedef enum { FFC_TRIANGLE = 2, FFC_TETRAHEDRON = 3 } ffc_cell; /* value = spat
 /* Arithmetic of the contraction A0 : G. J, its cofactors (adjugate) and det J are always
  * FP64: that is where a near-degenerate cell cancels. For FFC_FP64 the inverse
  * K = adj(J) / det J and G_K are FP64, and the contraction is FP64 multiply-adds or (Poisson,
- * the block algorithm, the adjoint) exact sums of 55- to 59-bit fixed-point products rounded
- * once, whose error is no larger; cells whose geometry factors differ by more than the fixed
- * point carries take the multiply-adds. For FFC_FP32 and the tensor-core precisions G_K
+ * the block algorithm, the adjoint) sums of 57- to 87-bit fixed-point products rounded once.
+ * Either way every entry is within a few ulps of the sum of its own |terms| A0 G, G taken
+ * down to the products behind the cofactors: the fixed point takes only cells where its units
+ * are small enough for each entry; cells whose factors (entries of K, coefficients, mu and
+ * lambda, the adjoint's dA) differ by more take the multiply-adds. Entries of A0 that are
+ * zero but for rounding may be rounded to 2^-59 of their row's largest. For FFC_FP32 and the tensor-core precisions G_K
  * is formed in FP32, the type it is rounded to anyway (the tensor cores further split it
  * into operand parts): the dense kernels form K in FP32 from the FP64 adjugate and
  * determinant (a well-conditioned step; cells with |det J| outside [1e-30, 1e30] divide

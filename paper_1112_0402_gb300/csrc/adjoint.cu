@@ -36,7 +36,7 @@
 // of few entries, it is. The contraction therefore also sums |A0||f| of each column in half
 // precision (three packed multiply-adds beside 18 integer ones) and takes a cell only where every
 // column's sum reaches THETA; there the worst error over dA of independent, rank-one, diagonal and
-// widely spread entries is 2e-16 to 1e-15 of the sum of |terms|, as with FP64 multiply-adds (2e-16
+// widely spread entries is 1e-16 to 8e-16 of the sum of |terms|, as with FP64 multiply-adds (2e-16
 // to 1e-15). P1's columns have three or four terms, and 3% of the cells of a rank-one dA would fail,
 // more than half of the warps: there dA is held in wide parts (fixed_point.cuh), and a cell is
 // taken where its nonzero entries are within 2^28 of one another. Other cells, and those whose dA

@@ -13,9 +13,10 @@
 // 2^(56 - 2B) of the scales each). Both sums stay within 63 bits for K 4^(B - 29) < 2^63:
 // B = 59 for K <= 7, B = 58 for K <= 31. Rounding the factors and dropping al gl costs at
 // most K 2^-B of 2^(ea + eg) in all; FP64 multiply-adds cost K 2^-53 of the partial sums.
-// The fixed point is thus the more accurate one wherever the partial sums are not more
-// than 2^(B - 53) below the scales, which the callers ensure by a condition on the cell
-// (its geometry factors of comparable size); other cells take the FP64 multiply-adds.
+// The fixed point is thus the more accurate one wherever an entry's own terms are not more
+// than 2^(B - 53) below the scales. The callers take a cell only where that holds for every
+// entry (each by its own rule, on the factors themselves); other cells take the FP64
+// multiply-adds. Factors a that are zero but for rounding are held to 2^-B of their row.
 #pragma once
 
 #include <cuda_runtime.h>

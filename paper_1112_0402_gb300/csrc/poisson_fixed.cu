@@ -8,8 +8,9 @@
 // the 6 FP64 ones) and about 25 other integer instructions. Now the latency of a chunk
 // (28% of the warps resident, issue 44%) and, for P1 and P2, the FP64 geometry bound the
 // tabulation (P4 0.59 of HBM), FP64 atomics the assembly. Measured, FP64 multiply-adds ->
-// fixed point: P4 tabulate of 384,000 tets 2645 -> 951 us, P3 assembly of 178,746 tets
-// (with zeroing) 546 -> 328 us, P2 tabulate of 1.05 M tets 790 -> 340 us.
+// fixed point: P4 tabulate of 384,000 tets 2645 -> 932 us, P3 assembly of 178,746 tets
+// (with zeroing) 546 -> 324 us, P2 tabulate of 1.05 M tets 790 -> 327 us; cells that take the
+// FP64 multiply-adds (stretched 1:64) P4 of 196,608 tets 1354 -> 745 us, P2 of 384,000 283 -> 161.
 //
 // One CTA takes tiles of E consecutive cells (persistent grid-stride loop):
 //   geometry  one thread per cell: FP64 J, K = J^-1, |det J| and the symmetric G_K
