@@ -40,8 +40,8 @@
 // to 1e-15). P1's columns have three or four terms, and 3% of the cells of a rank-one dA would fail,
 // more than half of the warps: there dA is held in wide parts (fixed_point.cuh), and a cell is
 // taken where its nonzero entries are within 2^28 of one another. Other cells, and those whose dA
-// is not finite or lies outside [2^-900, 2^900], take FP64 multiply-adds over all n^2 entries, L
-// lanes per cell.
+// is not finite or lies outside [2^-900, 2^900] (P1: [2^-700, 2^900]), take FP64 multiply-adds
+// over all n^2 entries, L lanes per cell.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(AdjCfg<D, Q>::WARPS * 32, AdjCfg<D, Q>::MIN_BL
 #pragma unroll
             for (int k = 0; k < NP; ++k) g[k] = 0.0;
             done = true;
-          } else if (top <= 900 && low >= -900 && top - low <= 28) {
+          } else if (top <= 900 && low >= FIX_CELL_MIN_WIDE && top - low <= 28) {
             FixAccWide acc[NP];
 #pragma unroll 2
             for (int u = 0; u < NE; ++u) {
@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(AdjCfg<D, Q>::WARPS * 32, AdjCfg<D, Q>::MIN_BL
               for (int k = l; k < NP; k += L) g[k] = 0.0;
               done = true;
             }
-          } else if (top <= 900 && top >= -900) {
+          } else if (top <= 900 && top >= FIX_CELL_MIN) {
             FixAcc acc[NP];
             __half2 mass[C::NH];  // sums of |A0||f| of two columns each
 #pragma unroll

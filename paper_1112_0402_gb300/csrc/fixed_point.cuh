@@ -38,6 +38,9 @@ __device__ __forceinline__ int fix_exponent_or(double x, int zero) { return fix_
 // Smallest exponent of a reference-tensor row: a row of zeros takes it, so that with cell
 // exponents from -900 up the constants of the conversions below keep normal exponents.
 constexpr int FIX_ROW_MIN = -100;
+// Smallest cell exponent with narrow and with wide factors: a wide sum can be as small as 2^-121
+// of its scales, and the exponent field of the conversion below must not pass zero there.
+constexpr int FIX_CELL_MIN = -900, FIX_CELL_MIN_WIDE = -700;
 
 // x 2^(B - e) rounded to the nearest integer (halves away from zero), |x| < 2^e, 52 <= B <= 59
 template <int B>

@@ -115,7 +115,7 @@ __device__ __forceinline__ void fixed_geometry(const FixedParams& p, long long e
   int top = hi;
 #pragma unroll
   for (int a = D; a < NP; ++a) top = max(top, fix_exponent(G[a]));
-  bool fixed = top <= 900 && lo >= -900 && hi - lo <= FIX_SPREAD;
+  bool fixed = top <= 900 && lo >= FIX_CELL_MIN && hi - lo <= FIX_SPREAD;
   // FP32 holds the off-diagonal entries' terms for cells of 1e-18 to 1e18; elsewhere they over-
   // or underflow, which fails the comparison
   float U[D][D], Ka[D][D];

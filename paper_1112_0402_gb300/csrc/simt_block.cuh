@@ -428,11 +428,11 @@ __device__ __forceinline__ void block_geometry_fixed(const SimtParams& p, long l
   for (int w = t; w < nc * PARTS; w += C::NT) {  // each thread its own parts again
     const int el = w / PARTS, part = w - el * PARTS;
     int top = Ts[el];
-    bool fixed = top <= 900 && top >= -900;
+    bool fixed = top <= 900 && top >= (C::WIDE ? FIX_CELL_MIN_WIDE : FIX_CELL_MIN);
     if constexpr (CONV) {
       if (top == -1022 && !(Zs[el] >> 31)) {  // H = 0: its parts are zero
         fixed = true;
-        top = -900;
+        top = FIX_CELL_MIN;
       }
       fixed = fixed && !(Xs[el] & BLOCK_FIX_NONE);
     } else {

@@ -224,3 +224,34 @@ def test_adjoint_upstream_spread(d, q, kind, regular):
 
     tol = (2 * n + 48) * ULP * gradient(S, np.maximum(U, np.abs(K)), 1)
     assert (np.abs(got - gradient(G, K, -1)) <= tol).all()
+
+
+@pytest.mark.parametrize("q", [1, 2, 3])
+@pytest.mark.parametrize("power", [-690, -705, -880, 880])
+def test_elasticity_far_from_one(q, power):
+    """mu and lambda times a power of two: the same tensors times that power, on either side of
+    the range of the fixed point, up to the two contractions' roundings (20 ulps of the largest)."""
+    import paper_1112_0402_gb300 as F
+
+    x = np.concatenate([_jittered(60), _aligned(7)])
+    args = _on_gpu(x)
+    A = F.tabulate(F.Form(F.ELASTICITY, F.TETRAHEDRON, q, 1.0, 1.25), *args).cpu().numpy()
+    scale = 2.0 ** power
+    B = F.tabulate(F.Form(F.ELASTICITY, F.TETRAHEDRON, q, scale, 1.25 * scale), *args).cpu().numpy() / scale
+    assert F.status_poll() == 0
+    assert (np.abs(B - A) <= 20 * ULP * np.abs(A).max((1, 2), keepdims=True)).all()
+
+
+@pytest.mark.parametrize("q", [1, 2, 4])
+@pytest.mark.parametrize("power", [-690, -705, -880, 880])
+def test_adjoint_far_from_one(q, power):
+    """The same of dA: the gradient scales, up to roundings (n^2 ulps of the largest component)."""
+    import paper_1112_0402_gb300 as F
+
+    form = F.Form(F.POISSON, F.TETRAHEDRON, q)
+    args = _on_gpu(_jittered(60))
+    dA = _upstream(1.0, form, 60)
+    got = [F.tabulate_adjoint(form, *args, torch.as_tensor(dA * s, device="cuda")).cpu().numpy().reshape(60, -1) / s
+           for s in (1.0, 2.0 ** power)]
+    assert F.status_poll() == 0
+    assert (np.abs(got[1] - got[0]) <= form.n_local ** 2 * 4 * ULP * np.abs(got[0]).max(1, keepdims=True)).all()
